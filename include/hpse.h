@@ -342,7 +342,8 @@ hpse_status hpse_setup_block_preconditioner(hpse_mesh *m);
  * candidate shape for the mesh's right-hand-side count on the factors it has
  * just built (variants 0-2 and 8 for >= 32 right-hand sides, 3-4 for 2..31,
  * 5-7 for one; 2, 4, 6 and 8 in FP32 only) and keeps the fastest.  Variants
- * 0-7 are FP32/FP64 CUDA-core tiles; variant 8 runs both products on the
+ * 2, 4 and 6 in FP32 and 3 and 5 in FP64 take both products in one pass over
+ * the factor, the others of 0-7 are CUDA-core tiles; variant 8 runs both products on the
  * tensor cores (tcgen05, 128 rows x 64 right-hand sides per CTA, each FP32
  * operand split into two TF32 parts, three MMAs per product, FP32
  * accumulation in tensor memory).  hpse_block_tile returns the chosen

@@ -48,6 +48,14 @@ def _generate():
                 with open(path, "w") as f:
                     f.write(text)
             units.append(path)
+    # the one-pass element-block products, one unit per precision
+    for prec, extra in (("f32", ""), ("f64", "#define BJP_F64\n")):
+        path = os.path.join(GEN, f"bj_pass_{prec}.cu")
+        text = f'{extra}#include "bj_pass.cu"\n'
+        if not os.path.exists(path) or open(path).read() != text:
+            with open(path, "w") as f:
+                f.write(text)
+        units.append(path)
     units.append(os.path.join(CSRC, "hpse.cu"))
     return units
 

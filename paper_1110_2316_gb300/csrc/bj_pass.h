@@ -1,0 +1,21 @@
+// bj_pass.h -- arguments of the element-block preconditioner's kernels and the
+// entry points of its one-pass product (bj_pass.cu, one unit per precision).
+#pragma once
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+struct BjArgs {
+  const int32_t *elems;    // element ids of one degree group
+  int32_t n_group;         // elements in the group
+  int32_t n;               // block size (W+1)^3
+  int32_t n_rhs;
+  int64_t ndof;            // stride between right-hand sides of a vector
+  const int64_t *dof_off;  // per element
+  const int64_t *blk_off;  // per element: offset of its packed block
+};
+
+// z = X^T (X r) for the group's elements and all right-hand sides (bj_pass.cuh).
+// X is read in whole 16-byte words: its allocation extends to the next one.
+// err: int32 on the device, set when a bounded wait expired.
+cudaError_t bj_pass_f32(const BjArgs &a, const float *X, const float *r, float *z, int32_t *err, cudaStream_t s);
+cudaError_t bj_pass_f64(const BjArgs &a, const double *X, const double *r, double *z, int32_t *err, cudaStream_t s);

@@ -15,15 +15,7 @@
 // definiteness once eps32 * kappa(A_ee) approaches 1).
 #pragma once
 
-struct BjArgs {
-  const int32_t *elems;    // element ids of one degree group
-  int32_t n_group;         // elements in the group
-  int32_t n;               // block size (W+1)^3
-  int32_t n_rhs;
-  int64_t ndof;            // stride between right-hand sides of a vector
-  const int64_t *dof_off;  // per element
-  const int64_t *blk_off;  // per element: offset of its packed block
-};
+#include "bj_pass.h"
 
 // offset of (i, j), j <= i, inside one packed block (n <= 1331: fits 32 bits)
 __device__ __forceinline__ int pk(int i, int j) { return i * (i + 1) / 2 + j; }
@@ -270,16 +262,23 @@ __global__ void k_bj_dot(BjArgs A, const T *z, const T *r, double *part) {
   if (threadIdx.x == 0) part[(int64_t)e * A.n_rhs + rr] = s;
 }
 
-// Tile shapes of the two triangular products (rows x right-hand sides per
-// CTA), picked per degree group and precision by timing the candidates of
-// the right-hand-side count on the actual factors (bj_candidates); variants
-// 2, 4 and 6 exceed 48 KB of static shared memory in FP64 and exist in FP32
-// only; variant 8 is the tensor-core form (bj_tc.cuh: 128 rows x 64
-// right-hand sides, 3xTF32), FP32 only, offered from 32 right-hand sides on.
+// Shapes of the two triangular products, picked per degree group and precision
+// by timing the candidates of the right-hand-side count on the actual factors
+// (bj_candidates).  bj_is_pass: both products in one pass over the factor
+// (bj_pass.cuh, bj_mma.cuh); the other variants below 8 are tiles of k_bj_tri
+// (rows x right-hand sides per CTA), variant 8 is the tensor-core form
+// (bj_tc.cuh: 128 rows x 64 right-hand sides, 3xTF32), offered from 32
+// right-hand sides on.  Variants 2, 4, 6 and 8 exist in FP32 only.
+// Config 2's factors (512 blocks of 729), one application, tiles -> pass:
+// FP32 270 -> 145 us (1 rhs), 468 -> 215 (4), 470 -> 242 (8), 871 -> 365 (16);
+// FP64 4820 -> 2417 us (4), 4810 -> 4600 (8), and for 8 blocks 400 -> 98 us
+// (4).  One FP64 right-hand side of many blocks stays with the 64 x 1 tile
+// (622 us against 767), of few blocks the pass is the faster (41 against 89).
 constexpr int BJ_NVAR = 9;
 constexpr int BJ_TC = 8;
 constexpr int BJ_TILE[BJ_NVAR][2] = {{64, 64}, {128, 32}, {256, 16}, {128, 8}, {256, 8},
                                      {128, 1}, {256, 1},  {64, 1},   {128, 64}};
+inline bool bj_is_pass(int v, bool fp32) { return fp32 ? (v == 2 || v == 4 || v == 6) : (v == 3 || v == 5); }
 inline bool bj_variant_ok(int v, bool fp32) {
   return v >= 0 && v < BJ_NVAR && (fp32 || (v != 2 && v != 4 && v != 6 && v != BJ_TC));
 }
@@ -299,19 +298,16 @@ static void bj_pair(const BjArgs &a, const T *X, const T *r, T *t, T *z, cudaStr
   k_bj_tri<T, true, TM, RT, TR, TC><<<g, TR * TC, 0, s>>>(a, X, t, z);
 }
 
-// z = X^T (X r) for the group with tile variant v; t: scratch vector of the same layout.
+// z = X^T (X r) for the group with a tile of k_bj_tri; t: scratch vector of the same layout.
 template <typename T>
 static cudaError_t bj_apply_group(const BjArgs &a, const T *X, const T *r, T *t, T *z, cudaStream_t s, int v) {
   if (a.n_group == 0) return cudaSuccess;
   if (v == 0) bj_pair<T, 64, 64, 16, 16>(a, X, r, t, z, s);
   else if (v == 1) bj_pair<T, 128, 32, 32, 8>(a, X, r, t, z, s);
-  else if (v == 3) bj_pair<T, 128, 8, 64, 4>(a, X, r, t, z, s);
-  else if (v == 5) bj_pair<T, 128, 1, 128, 1>(a, X, r, t, z, s);
   else if (v == 7) bj_pair<T, 64, 1, 64, 1>(a, X, r, t, z, s);
   else if constexpr (sizeof(T) == 4) {
-    if (v == 2) bj_pair<T, 256, 16, 64, 4>(a, X, r, t, z, s);
-    else if (v == 4) bj_pair<T, 256, 8, 128, 2>(a, X, r, t, z, s);
-    else if (v == 6) bj_pair<T, 256, 1, 256, 1>(a, X, r, t, z, s);
+    if (v == 3) bj_pair<T, 128, 8, 64, 4>(a, X, r, t, z, s);
+    else if (v == 5) bj_pair<T, 128, 1, 128, 1>(a, X, r, t, z, s);
     else return cudaErrorInvalidValue;
   } else {
     return cudaErrorInvalidValue;

@@ -1152,6 +1152,11 @@ static hpse_status bj_products(hpse_mesh *m, const Group &g, const BjArgs &a, co
   if constexpr (sizeof(T) == 4) {
     if (v == BJ_TC) return bj_tc_pair(m, g, a.n_rhs, r, t, z, s);
   }
+  if (bj_is_pass(v, sizeof(T) == 4)) {
+    if constexpr (sizeof(T) == 4) CK(bj_pass_f32(a, X, r, z, m->d_bjt_err.as<int32_t>(), s));
+    else CK(bj_pass_f64(a, X, r, z, m->d_bjt_err.as<int32_t>(), s));
+    return HPSE_OK;
+  }
   CK(bj_apply_group<T>(a, X, r, t, z, s, v));
   return HPSE_OK;
 }
@@ -1222,8 +1227,9 @@ static hpse_status launch_bj_all(hpse_mesh *m, int mode, const PrecArgsT<T> &b, 
       // FP32 solve, FP64 factor: convert, apply, convert back
       k_bj_cvt<T, double><<<items, 128, 0, gs>>>(a, rin, m->bj_r64.as<double>());
       CK(cudaGetLastError());
-      CK(bj_apply_group<double>(a, m->d_bj64.as<double>(), m->bj_r64.as<double>(), m->bj_t64.as<double>(),
-                                m->bj_z64.as<double>(), gs, m->bj_var[g.W][0]));
+      hpse_status st = bj_products<double>(m, g, a, m->d_bj64.as<double>(), m->bj_r64.as<double>(),
+                                           m->bj_t64.as<double>(), m->bj_z64.as<double>(), gs, m->bj_var[g.W][0]);
+      if (st != HPSE_OK) return st;
       k_bj_cvt<double, T><<<items, 128, 0, gs>>>(a, m->bj_z64.as<double>(), b.zout);
       CK(cudaGetLastError());
       g_launches += 4;
@@ -2877,8 +2883,9 @@ extern "C" hpse_status hpse_setup_block_preconditioner(hpse_mesh *m) {
   CK(upload(m->d_bj_off, off));
   DevBuf blk;
   if (blk.alloc(std::max<int64_t>(total, 1) * sizeof(double)) != cudaSuccess) return HPSE_ERR_OOM;
-  if (m->d_bj64.alloc(std::max<int64_t>(total, 1) * sizeof(double)) != cudaSuccess) return HPSE_ERR_OOM;
-  if (m->d_bj32.alloc(std::max<int64_t>(total, 1) * sizeof(float)) != cudaSuccess) return HPSE_ERR_OOM;
+  // 16 bytes more: the one-pass product copies whole 16-byte words
+  if (m->d_bj64.alloc(std::max<int64_t>(total, 1) * sizeof(double) + 16) != cudaSuccess) return HPSE_ERR_OOM;
+  if (m->d_bj32.alloc(std::max<int64_t>(total, 1) * sizeof(float) + 16) != cudaSuccess) return HPSE_ERR_OOM;
   const size_t nv = (size_t)m->n_rhs * m->ndof;
   if (m->bj_t64.alloc(std::max<size_t>(nv, 1) * sizeof(double)) != cudaSuccess) return HPSE_ERR_OOM;
   if (m->bj_t32.alloc(std::max<size_t>(nv, 1) * sizeof(float)) != cudaSuccess) return HPSE_ERR_OOM;
@@ -2935,6 +2942,8 @@ extern "C" hpse_status hpse_setup_block_preconditioner(hpse_mesh *m) {
   int32_t h_fail = 0;
   CK(cudaMemcpy(&h_fail, fail.p, sizeof(int32_t), cudaMemcpyDeviceToHost));
   if (h_fail) return HPSE_ERR_BREAKDOWN;
+  if (!m->d_bjt_err.p) CK(m->d_bjt_err.alloc(sizeof(int32_t)));
+  CK(cudaMemset(m->d_bjt_err.p, 0, sizeof(int32_t)));
   // tensor-core form (a candidate from 32 right-hand sides on): FP32 tiles of
   // X and X^T per element
   m->d_bjt = DevBuf();
@@ -2947,8 +2956,6 @@ extern "C" hpse_status hpse_setup_block_preconditioner(hpse_mesh *m) {
     }
     if (m->d_bjt.alloc((size_t)toff[E] * sizeof(float)) != cudaSuccess) return HPSE_ERR_OOM;
     CK(upload(m->d_bjt_off, toff));
-    if (!m->d_bjt_err.p) CK(m->d_bjt_err.alloc(sizeof(int32_t)));
-    CK(cudaMemset(m->d_bjt_err.p, 0, sizeof(int32_t)));
     CK(raise_smem((const void *)k_bj_tc<false>, m->device, BJT_SMEM));
     CK(raise_smem((const void *)k_bj_tc<true>, m->device, BJT_SMEM));
     for (size_t gi = 0; gi < m->groups.size(); ++gi) {
@@ -2987,22 +2994,20 @@ extern "C" hpse_status hpse_setup_block_preconditioner(hpse_mesh *m) {
           float ms = 0.0f;
           for (int rep = 0; rep < 4; ++rep) {
             if (rep == 1) CK(cudaEventRecord(e0, s));
-            if (pi == 0)
-              CK(bj_apply_group<double>(ba, m->d_bj64.as<double>(), tin.as<double>(), m->bj_t64.as<double>(),
-                                        tout.as<double>(), s, v));
-            else {
-              const hpse_status st = bj_products<float>(m, g, ba, m->d_bj32.as<float>(), tin.as<float>(),
-                                                        m->bj_t32.as<float>(), tout.as<float>(), s, v);
-              if (st != HPSE_OK) return st;
-            }
+            const hpse_status st =
+                pi == 0 ? bj_products<double>(m, g, ba, m->d_bj64.as<double>(), tin.as<double>(),
+                                              m->bj_t64.as<double>(), tout.as<double>(), s, v)
+                        : bj_products<float>(m, g, ba, m->d_bj32.as<float>(), tin.as<float>(), m->bj_t32.as<float>(),
+                                             tout.as<float>(), s, v);
+            if (st != HPSE_OK) return st;
             g_launches += 2;
           }
           CK(cudaEventRecord(e1, s));
           CK(cudaEventSynchronize(e1));
           CK(cudaEventElapsedTime(&ms, e0, e1));
           ms /= 3.0f;
-          if (v == BJ_TC) {
-            // a tensor-core product whose bounded wait expired is not a candidate
+          if (v == BJ_TC || bj_is_pass(v, pi == 1)) {
+            // a product whose bounded wait expired is not a candidate
             int32_t h_err = 0;
             CK(cudaMemcpy(&h_err, m->d_bjt_err.p, sizeof(int32_t), cudaMemcpyDeviceToHost));
             if (h_err) continue;
@@ -3036,9 +3041,10 @@ extern "C" hpse_status hpse_setup_block_preconditioner(hpse_mesh *m) {
     for (size_t gi = 0; gi < m->groups.size(); ++gi) {
       const Group &g = m->groups[gi];
       const BjArgs ba = bj_args(m, g, m->n_rhs);
-      CK(bj_apply_group<double>(ba, m->d_bj64.as<double>(), v64.as<double>(), m->bj_t64.as<double>(),
-                                z64.as<double>(), s, m->bj_var[g.W][0]));
-      const hpse_status st = bj_products<float>(m, g, ba, m->d_bj32.as<float>(), v32.as<float>(),
+      hpse_status st = bj_products<double>(m, g, ba, m->d_bj64.as<double>(), v64.as<double>(), m->bj_t64.as<double>(),
+                                           z64.as<double>(), s, m->bj_var[g.W][0]);
+      if (st != HPSE_OK) return st;
+      st = bj_products<float>(m, g, ba, m->d_bj32.as<float>(), v32.as<float>(),
                                                 m->bj_t32.as<float>(), z32.as<float>(), s, m->bj_var[g.W][1]);
       if (st != HPSE_OK) return st;
       CK(cudaMemsetAsync(acc.p, 0, 2 * sizeof(double), s));
