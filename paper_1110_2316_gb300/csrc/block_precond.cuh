@@ -7,8 +7,7 @@
 // Set-up (FP64): A_ee is probed column by column with the operator kernel in
 // self-only mode (neighbour traces taken as zero), gathered into packed
 // lower-triangular storage (row i holds columns 0..i at offset i(i+1)/2),
-// factored A_ee = L L^T (right-looking Cholesky, one CTA per block) and
-// X = L^{-1} is formed row by row.  The preconditioner is z = X^T (X r): two
+// factored A_ee = L L^T and X = L^{-1} is formed, both in 64 x 64 tiles.  The preconditioner is z = X^T (X r): two
 // triangular products, kept in FP64 and rounded to FP32.  Storing the factor
 // rather than A_ee^{-1} keeps the FP32 operator X~^T X~ symmetric positive
 // definite whatever the rounding of X (A_ee^{-1} itself rounded to FP32 loses
@@ -39,71 +38,220 @@ __global__ void k_bj_gather(BjArgs A, int j0, int nc, const double *y, double *b
   for (int i = j + threadIdx.x; i < A.n; i += blockDim.x) B[pk(i, j)] = y[base + i];
 }
 
-// in-place Cholesky A = L L^T of each packed block; fail[0] set (block index
-// + 1) on a non-positive pivot, the block is then left partly factored.
-// Dynamic shared memory: n doubles.
-__global__ void __launch_bounds__(256) k_bj_chol(BjArgs A, double *blk, int32_t *fail) {
-  extern __shared__ double colk[];
-  __shared__ double s_inv;
+// ---------------------------------------------------------------------------
+// Factorisation A_ee = L L^T and X = L^{-1} in 64 x 64 tiles of the packed
+// blocks, every step one launch over all elements of the group:
+//   for block column p: k_bj_diag   L_pp by columns, X_pp = L_pp^{-1}
+//                       k_bj_panel  L_ip = A_ip X_pp^T,            i > p
+//                       k_bj_syrk   A_ij -= L_ip L_jp^T,       i >= j > p
+//   for block row i:    k_bj_xrow   X_ij = -X_ii sum_{j <= m < i} L_im X_mj
+// Bound by the FP64 pipe (2 x n^3 / 6 multiply-adds per block).  One CTA per
+// block, column by column through global memory, took 119 + 41 ms for 64
+// blocks of 729: the tiles spread a block over the SMs and read each operand
+// once per 64 multiply-adds (20 ms, of which 13 are the pipe's).
+// fail[0] is set (block index + 1) on a non-positive or non-finite pivot; the
+// factorisation then goes on with pivot 1 and its result is not used.
+// ---------------------------------------------------------------------------
+constexpr int BJB = 64;                      // tile edge
+constexpr int BJB_LD = BJB + 1;              // leading dimension of a whole tile in shared memory
+constexpr int BJB_KC = 32;                   // K chunk of the tile products
+constexpr size_t BJB_SMEM2 = 2 * (size_t)BJB * BJB_LD * sizeof(double);
+constexpr size_t BJB_SMEM_X = ((size_t)BJB * BJB_LD + 2 * (size_t)BJB * (BJB_KC + 1)) * sizeof(double);
+
+__global__ void __launch_bounds__(256) k_bj_diag(BjArgs A, int p, double *blk, double *xout, int32_t *fail) {
+  extern __shared__ double bjb_sm[];
+  double *L = bjb_sm, *V = bjb_sm + BJB * BJB_LD;
+  __shared__ double s_inv[BJB];
   __shared__ int s_bad;
-  const int e = A.elems[blockIdx.x], n = A.n;
-  double *L = blk + A.blk_off[e];
-  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, w = tid >> 5, nw = nt >> 5;
+  const int e = A.elems[blockIdx.x], n = A.n, i0 = BJB * p, m = min(BJB, n - i0);
+  double *B = blk + A.blk_off[e], *X = xout + A.blk_off[e];
+  const int tid = threadIdx.x;
+  for (int t = tid; t < BJB * BJB; t += 256) {
+    const int i = t / BJB, j = t - i * BJB;
+    L[i * BJB_LD + j] = (i < m && j <= i) ? B[pk(i0 + i, i0 + j)] : 0.0;
+    V[i * BJB_LD + j] = i == j ? 1.0 : 0.0;
+  }
   if (tid == 0) s_bad = 0;
-  for (int k = 0; k < n; ++k) {
+  __syncthreads();
+  const int ri = tid >> 2, rc = tid & 3;
+  for (int k = 0; k < m; ++k) {
     if (tid == 0) {
-      double d = L[pk(k, k)];
+      double d = L[k * BJB_LD + k];
       if (!(d > 0.0) || !isfinite(d)) {
         s_bad = 1;
         d = 1.0;
       }
       d = sqrt(d);
-      L[pk(k, k)] = d;
-      s_inv = 1.0 / d;
+      L[k * BJB_LD + k] = d;
+      s_inv[k] = 1.0 / d;
     }
     __syncthreads();
-    if (s_bad) break;
-    for (int i = k + 1 + tid; i < n; i += nt) {
-      const double v = L[pk(i, k)] * s_inv;
-      L[pk(i, k)] = v;
-      colk[i] = v;
+    if (tid > k && tid < m) L[tid * BJB_LD + k] *= s_inv[k];
+    __syncthreads();
+    if (ri > k && ri < m) {
+      const double li = L[ri * BJB_LD + k];
+      for (int j = k + 1 + rc; j <= ri; j += 4) L[ri * BJB_LD + j] -= li * L[j * BJB_LD + k];
     }
     __syncthreads();
-    // trailing update of rows i > k, columns k < j <= i: one warp per row
-    for (int i = k + 1 + w; i < n; i += nw) {
-      const double li = colk[i];
-      double *Li = L + pk(i, 0);
-      for (int j = k + 1 + lane; j <= i; j += 32) Li[j] -= li * colk[j];
+  }
+  // X_pp by forward substitution on the identity, row by row
+  for (int k = 0; k < m; ++k) {
+    if (tid <= k) V[k * BJB_LD + tid] *= s_inv[k];
+    __syncthreads();
+    if (ri > k && ri < m) {
+      const double li = L[ri * BJB_LD + k];
+      for (int j = rc; j <= k; j += 4) V[ri * BJB_LD + j] -= li * V[k * BJB_LD + j];
     }
     __syncthreads();
+  }
+  for (int t = tid; t < BJB * BJB; t += 256) {
+    const int i = t / BJB, j = t - i * BJB;
+    if (i < m && j <= i) {
+      B[pk(i0 + i, i0 + j)] = L[i * BJB_LD + j];
+      X[pk(i0 + i, i0 + j)] = V[i * BJB_LD + j];
+    }
   }
   if (tid == 0 && s_bad) atomicCAS(fail, 0, blockIdx.x + 1);
 }
 
-// X = L^{-1} (packed lower), row by row: X_ii = 1 / L_ii and, for j < i,
-// X_ij = -(sum_{j <= m < i} L_im X_mj) / L_ii.  Dynamic shared memory: n doubles.
-__global__ void __launch_bounds__(256) k_bj_trinv(BjArgs A, const double *blk, double *xout) {
-  extern __shared__ double lrow[];
-  const int e = A.elems[blockIdx.x], n = A.n;
-  const double *L = blk + A.blk_off[e];
-  double *X = xout + A.blk_off[e];
-  const int tid = threadIdx.x, nt = blockDim.x;
-  for (int i = 0; i < n; ++i) {
-    for (int m = tid; m <= i; m += nt) lrow[m] = L[pk(i, m)];
-    __syncthreads();
-    const double inv = 1.0 / lrow[i];
-    // columns in chunks of nt; rows m of X are read in order, so at each m
-    // the active threads read consecutive addresses of row m
-    for (int j0 = 0; j0 <= i; j0 += nt) {
-      const int j = j0 + tid;
-      double s = 0.0;
-      for (int m = j0; m < i; ++m)
-        if (m >= j) s += lrow[m] * X[pk(m, j)];
-      if (j < i) X[pk(i, j)] = -s * inv;
-      else if (j == i) X[pk(i, i)] = inv;
+// rows r0.. (BJB of them), columns c0 .. c0 + BJB_KC of a packed lower triangle
+// into S[row][BJB_KC + 1]; zero above the diagonal and beyond n
+__device__ __forceinline__ void bjb_load(const double *B, int n, int r0, int c0, double *S) {
+  for (int t = threadIdx.x; t < BJB * BJB_KC; t += 256) {
+    const int i = t / BJB_KC, j = t - i * BJB_KC;
+    const int r = r0 + i, c = c0 + j;
+    S[i * (BJB_KC + 1) + j] = (r < n && c <= r) ? B[pk(r, c)] : 0.0;
+  }
+}
+// the same transposed: rows c0 .. c0 + BJB_KC, columns r0.. into S[column][row]
+__device__ __forceinline__ void bjb_load_t(const double *B, int n, int r0, int c0, double *S) {
+  for (int t = threadIdx.x; t < BJB * BJB_KC; t += 256) {
+    const int j = t / BJB, i = t - j * BJB;
+    const int r = c0 + j, c = r0 + i;
+    S[i * (BJB_KC + 1) + j] = (r < n && c <= r) ? B[pk(r, c)] : 0.0;
+  }
+}
+// acc[a][b] += sum_k P[ty + 16 a][k] Q[tx + 16 b][k] over one chunk
+__device__ __forceinline__ void bjb_mac(const double *P, int ldp, const double *Q, double (&acc)[4][4]) {
+  const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
+#pragma unroll 4
+  for (int k = 0; k < BJB_KC; ++k) {
+    double p[4], q[4];
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+      p[a] = P[(ty + 16 * a) * ldp + k];
+      q[a] = Q[(tx + 16 * a) * (BJB_KC + 1) + k];
     }
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+      for (int b = 0; b < 4; ++b) acc[a][b] += p[a] * q[b];
+  }
+}
+
+// L_ip = A_ip X_pp^T.  grid: n_group * (blocks below p)
+__global__ void __launch_bounds__(256) k_bj_panel(BjArgs A, int p, double *blk, const double *xin) {
+  __shared__ double P[BJB * (BJB_KC + 1)], Q[BJB * (BJB_KC + 1)];
+  const int n = A.n, nt = (n + BJB - 1) / BJB - 1 - p;
+  const int ge = blockIdx.x / nt, i = p + 1 + blockIdx.x - ge * nt;
+  const int e = A.elems[ge];
+  double *B = blk + A.blk_off[e];
+  const double *X = xin + A.blk_off[e];
+  double acc[4][4] = {};
+  for (int c = 0; c < BJB; c += BJB_KC) {
+    bjb_load(B, n, BJB * i, BJB * p + c, P);
+    bjb_load(X, n, BJB * p, BJB * p + c, Q);
+    __syncthreads();
+    bjb_mac(P, BJB_KC + 1, Q, acc);
     __syncthreads();
   }
+  const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+      const int r = BJB * i + ty + 16 * a;
+      if (r < n) B[pk(r, BJB * p + tx + 16 * b)] = acc[a][b];
+    }
+}
+
+// A_ij -= L_ip L_jp^T on the trailing tiles.  grid: n_group * T (T + 1) / 2, T = blocks below p
+__global__ void __launch_bounds__(256) k_bj_syrk(BjArgs A, int p, double *blk) {
+  __shared__ double P[BJB * (BJB_KC + 1)], Q[BJB * (BJB_KC + 1)];
+  const int n = A.n, nt = (n + BJB - 1) / BJB - 1 - p, tiles = nt * (nt + 1) / 2;
+  const int ge = blockIdx.x / tiles, t = blockIdx.x - ge * tiles;
+  int ti = 0;
+  while ((ti + 1) * (ti + 2) / 2 <= t) ++ti;
+  const int i = p + 1 + ti, j = p + 1 + t - ti * (ti + 1) / 2;
+  double *B = blk + A.blk_off[A.elems[ge]];
+  double acc[4][4] = {};
+  for (int c = 0; c < BJB; c += BJB_KC) {
+    bjb_load(B, n, BJB * i, BJB * p + c, P);
+    bjb_load(B, n, BJB * j, BJB * p + c, Q);
+    __syncthreads();
+    bjb_mac(P, BJB_KC + 1, Q, acc);
+    __syncthreads();
+  }
+  const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+      const int r = BJB * i + ty + 16 * a, c = BJB * j + tx + 16 * b;
+      if (r < n && c <= r) B[pk(r, c)] -= acc[a][b];
+    }
+}
+
+// X_ij = -X_ii sum_{j <= m < i} L_im X_mj.  grid: n_group * i (j = 0, the longest sum, first)
+__global__ void __launch_bounds__(256) k_bj_xrow(BjArgs A, int i, const double *blk, double *xout) {
+  extern __shared__ double bjb_sm[];
+  double *S = bjb_sm, *P = bjb_sm + BJB * BJB_LD, *Q = P + BJB * (BJB_KC + 1);
+  const int n = A.n;
+  const int j = blockIdx.x / A.n_group, ge = blockIdx.x - j * A.n_group;
+  const int e = A.elems[ge];
+  const double *B = blk + A.blk_off[e];
+  double *X = xout + A.blk_off[e];
+  double acc[4][4] = {};
+  for (int k = BJB * j; k < BJB * i; k += BJB_KC) {
+    bjb_load(B, n, BJB * i, k, P);
+    bjb_load_t(X, n, BJB * j, k, Q);
+    __syncthreads();
+    bjb_mac(P, BJB_KC + 1, Q, acc);
+    __syncthreads();
+  }
+  // the sum transposed (S[column][row]) as the right factor of X_ii S
+  const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int b = 0; b < 4; ++b) S[(tx + 16 * b) * BJB_LD + ty + 16 * a] = acc[a][b];
+  double out[4][4] = {};
+  for (int c = 0; c < BJB; c += BJB_KC) {
+    __syncthreads();
+    bjb_load(X, n, BJB * i, BJB * i + c, P);
+    __syncthreads();
+    // P: X_ii rows; S read as rows tx + 16 b at columns c + k
+#pragma unroll 4
+    for (int k = 0; k < BJB_KC; ++k) {
+      double p[4], q[4];
+#pragma unroll
+      for (int a = 0; a < 4; ++a) {
+        p[a] = P[(ty + 16 * a) * (BJB_KC + 1) + k];
+        q[a] = S[(tx + 16 * a) * BJB_LD + c + k];
+      }
+#pragma unroll
+      for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int b = 0; b < 4; ++b) out[a][b] += p[a] * q[b];
+    }
+  }
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+      const int r = BJB * i + ty + 16 * a;
+      if (r < n) X[pk(r, BJB * j + tx + 16 * b)] = -out[a][b];
+    }
 }
 
 template <typename T>

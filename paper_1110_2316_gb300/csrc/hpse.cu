@@ -2925,14 +2925,28 @@ extern "C" hpse_status hpse_setup_block_preconditioner(hpse_mesh *m) {
       CK(cudaGetLastError());
       g_launches += 3;
     }
-    const size_t sm = (size_t)n * sizeof(double);
-    CK(raise_smem((const void *)k_bj_chol, m->device, (size_t)std::max<size_t>(sm, 1)));
-    CK(raise_smem((const void *)k_bj_trinv, m->device, (size_t)std::max<size_t>(sm, 1)));
-    k_bj_chol<<<g.n, 256, sm, s>>>(ba, blk.as<double>(), fail.as<int32_t>());
-    CK(cudaGetLastError());
-    k_bj_trinv<<<g.n, 256, sm, s>>>(ba, blk.as<double>(), m->d_bj64.as<double>());
-    CK(cudaGetLastError());
-    g_launches += 2;
+    // A = L L^T, X = L^{-1} by 64 x 64 tiles
+    const int nb = (n + BJB - 1) / BJB;
+    CK(raise_smem((const void *)k_bj_diag, m->device, BJB_SMEM2));
+    CK(raise_smem((const void *)k_bj_xrow, m->device, BJB_SMEM_X));
+    double *Lb = blk.as<double>(), *Xb = m->d_bj64.as<double>();
+    for (int p = 0; p < nb; ++p) {
+      const int T = nb - 1 - p;
+      k_bj_diag<<<g.n, 256, BJB_SMEM2, s>>>(ba, p, Lb, Xb, fail.as<int32_t>());
+      CK(cudaGetLastError());
+      ++g_launches;
+      if (T == 0) continue;
+      k_bj_panel<<<g.n * T, 256, 0, s>>>(ba, p, Lb, Xb);
+      CK(cudaGetLastError());
+      k_bj_syrk<<<g.n * (T * (T + 1) / 2), 256, 0, s>>>(ba, p, Lb);
+      CK(cudaGetLastError());
+      g_launches += 2;
+    }
+    for (int i = 1; i < nb; ++i) {
+      k_bj_xrow<<<g.n * i, 256, BJB_SMEM_X, s>>>(ba, i, Lb, Xb);
+      CK(cudaGetLastError());
+      ++g_launches;
+    }
   }
   if (total > 0) {
     k_bj_convert<float><<<1024, 256, 0, s>>>(m->d_bj64.as<double>(), m->d_bj32.as<float>(), total);
