@@ -59,17 +59,23 @@ size_t apply_smem_fn(int coef) {
 
 int apply_max_threads_fn(int) { return NT; }
 
+template <int MODE, int ITEMS>
+cudaError_t launch_precond_t(const void *args, int n_items, cudaStream_t s) {
+  typedef PcLayout<ITEMS> L;
+  const int grid = (n_items + ITEMS - 1) / ITEMS;
+  k_precond<MODE, ITEMS><<<grid, L::NTH, L::BYTES, s>>>(*static_cast<const PrecArgs *>(args));
+  return cudaGetLastError();
+}
+
 cudaError_t precond_fn(int mode, const void *args, int n_items, int threads, cudaStream_t s) {
   if (n_items <= 0) return cudaSuccess;
-  (void)threads;  // CTA shape fixed at compile time: PC_ITEMS items of PC_TPI threads
-  const int grid = (n_items + PC_ITEMS - 1) / PC_ITEMS;
+  (void)threads;  // CTA shape fixed at compile time: items of PC_TPI threads
+  const bool few = PC_ITEMS > 1 && n_items < PC_FEW;
   if (mode == MODE_PLAIN)
-    k_precond<MODE_PLAIN><<<grid, PC_NT, PC_BYTES, s>>>(*static_cast<const PrecArgs *>(args));
-  else if (mode == MODE_PCG)
-    k_precond<MODE_PCG><<<grid, PC_NT, PC_BYTES, s>>>(*static_cast<const PrecArgs *>(args));
-  else
-    return cudaErrorInvalidValue;
-  return cudaGetLastError();
+    return few ? launch_precond_t<MODE_PLAIN, 1>(args, n_items, s) : launch_precond_t<MODE_PLAIN, PC_ITEMS>(args, n_items, s);
+  if (mode == MODE_PCG)
+    return few ? launch_precond_t<MODE_PCG, 1>(args, n_items, s) : launch_precond_t<MODE_PCG, PC_ITEMS>(args, n_items, s);
+  return cudaErrorInvalidValue;
 }
 
 template <int COEF, int MODE>
@@ -182,11 +188,11 @@ cudaError_t upload_fn(const double *pk) {
   if ((e2 = set_smem_attr_gen<MODE_TRANSPOSE>()) != cudaSuccess) return e2;
   if ((e2 = set_smem_attr_ibp<COEF_LAPLACE>()) != cudaSuccess) return e2;
   if ((e2 = set_smem_attr_ibp<COEF_SCALAR>()) != cudaSuccess) return e2;
-  if ((e2 = cudaFuncSetAttribute(k_precond<MODE_PLAIN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)PC_BYTES)) != cudaSuccess)
+  if ((e2 = cudaFuncSetAttribute(k_precond<MODE_PLAIN, PC_ITEMS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)PcLayout<PC_ITEMS>::BYTES)) != cudaSuccess)
     return e2;
-  if ((e2 = cudaFuncSetAttribute(k_precond<MODE_PCG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)PC_BYTES)) != cudaSuccess)
+  if ((e2 = cudaFuncSetAttribute(k_precond<MODE_PCG, PC_ITEMS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)PcLayout<PC_ITEMS>::BYTES)) != cudaSuccess)
     return e2;
   return cudaSuccess;
 }

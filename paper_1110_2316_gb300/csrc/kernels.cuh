@@ -1668,17 +1668,25 @@ __global__ void __launch_bounds__(NT, APPLY_MINB) k_apply(const ApplyArgs A) {
 // writes the partial sums r.r and r.z.
 // ---------------------------------------------------------------------------
 // Preconditioner CTAs hold several (element, rhs) items; each item owns
-// PC_TPI threads (one per line of P nodes, whole warps).
+// PC_TPI threads (one per line of P nodes, whole warps).  Launches whose items
+// would fill fewer CTAs than twice the SMs take one item per CTA instead: an
+// FP64 item alone is bound by its SM's FP64 pipe (two lanes per clock), so six
+// items on one SM and none on the next cost six times (128 FP64 items of W = 6:
+// 45 -> 19 us, 1,024: 84 -> 53 us; FP32 stays at the launch's latency).
 constexpr int PC_TPI = PAD32(P2);
 constexpr int PC_ITEMS_RAW = 384 / PC_TPI;
 constexpr int PC_ITEMS = PC_ITEMS_RAW < 1 ? 1 : (PC_ITEMS_RAW > 8 ? 8 : PC_ITEMS_RAW);
-constexpr int PC_NT = PC_ITEMS * PC_TPI;
+constexpr int PC_FEW = 304 * PC_ITEMS;
 constexpr int PC_WARPS_PER_ITEM = PC_TPI / 32;
 // per item: two P^3 blocks; then the reduction buffer; then per item the x3
 // eigenbasis and eigenvalues of the C* form (edge neighbourhood)
-constexpr size_t PC_RED_OFF = (size_t)PC_ITEMS * 2 * P3 * sizeof(real);
-constexpr size_t PC_Z_OFF = PC_RED_OFF + (size_t)(PC_NT / 32) * 2 * sizeof(double);
-constexpr size_t PC_BYTES = PC_Z_OFF + (size_t)PC_ITEMS * (P2 + P) * sizeof(real);
+template <int ITEMS>
+struct PcLayout {
+  static constexpr int NTH = ITEMS * PC_TPI;
+  static constexpr size_t RED_OFF = (((size_t)ITEMS * 2 * P3 * sizeof(real) + 15) / 16) * 16;
+  static constexpr size_t Z_OFF = RED_OFF + (size_t)(NTH / 32) * 2 * sizeof(double);
+  static constexpr size_t BYTES = Z_OFF + (size_t)ITEMS * (P2 + P) * sizeof(real);
+};
 
 // out = (S^T or S) applied along `axis` of one P x P x P block (x fastest);
 // thread lt of the item handles line lt (no loop: PC_TPI >= P^2 lines)
@@ -1749,18 +1757,19 @@ __device__ __forceinline__ double item_sum(double v, double *red, int warp_in_ct
   return t;
 }
 
-template <int MODE>
-__global__ void __launch_bounds__(PC_NT) k_precond(const PrecArgs A) {
+template <int MODE, int ITEMS>
+__global__ void __launch_bounds__(PcLayout<ITEMS>::NTH) k_precond(const PrecArgs A) {
+  typedef PcLayout<ITEMS> L;
   extern __shared__ __align__(16) unsigned char pc_raw[];
   const int sub = threadIdx.x / PC_TPI;  // item within the CTA (warp-uniform)
   const int lt = threadIdx.x - sub * PC_TPI;
   real *s0 = reinterpret_cast<real *>(pc_raw) + (size_t)sub * 2 * P3;
   real *s1 = s0 + P3;
-  double *red = reinterpret_cast<double *>(pc_raw + PC_RED_OFF);
-  real *sz = reinterpret_cast<real *>(pc_raw + PC_Z_OFF) + (size_t)sub * (P2 + P);
+  double *red = reinterpret_cast<double *>(pc_raw + L::RED_OFF);
+  real *sz = reinterpret_cast<real *>(pc_raw + L::Z_OFF) + (size_t)sub * (P2 + P);
   const bool cstar = A.zeig != nullptr;
   __shared__ real smu[P];
-  const int item = blockIdx.x * PC_ITEMS + sub;
+  const int item = blockIdx.x * ITEMS + sub;
   const bool valid = item < A.n_group * A.n_rhs;
   const int ge = valid ? item / A.n_rhs : 0;
   const int rr = valid ? item - ge * A.n_rhs : 0;
