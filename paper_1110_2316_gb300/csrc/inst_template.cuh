@@ -106,11 +106,19 @@ cudaError_t upload_fn(const double *pk) {
         t.FO[m][q * HPE + j] = (real)(mid ? 0.0 : 0.5 * (b[q * P + j] - b[q * P + P - 1 - j]));
       }
   }
+  auto pair = [](real x, real y) {
+    real2 v;
+    v.x = x;
+    v.y = y;
+    return v;
+  };
   for (int i = 0; i < P * HPE; ++i) {
-    t.XE[0][i] = make_float2((float)t.FE[0][i], (float)t.FE[0][i]);
-    t.XE[1][i] = make_float2((float)t.FE[0][i], (float)t.FE[2][i]);
-    t.XO[0][i] = make_float2((float)t.FO[0][i], (float)t.FO[0][i]);
-    t.XO[1][i] = make_float2((float)t.FO[0][i], (float)t.FO[2][i]);
+    t.XE[0][i] = pair(t.FE[0][i], t.FE[0][i]);
+    t.XE[1][i] = pair(t.FE[0][i], t.FE[2][i]);
+    t.XE[2][i] = pair(t.FE[1][i], t.FE[1][i]);
+    t.XO[0][i] = pair(t.FO[0][i], t.FO[0][i]);
+    t.XO[1][i] = pair(t.FO[0][i], t.FO[2][i]);
+    t.XO[2][i] = pair(t.FO[1][i], t.FO[1][i]);
   }
   const double *pD = pk + o;
   for (int i = 0; i < P2; ++i) t.D[i] = (real)pk[o++];

@@ -48,6 +48,14 @@ constexpr int QP2 = Q * P * P;
 constexpr int Q2P = Q * Q * P;
 
 typedef REAL real;
+// two values handled together: FP32 pairs go through the packed FMA
+#if defined(HPSE_DOUBLE)
+typedef double2 real2;
+__device__ __forceinline__ real2 mk2(real x, real y) { return make_double2(x, y); }
+#else
+typedef float2 real2;
+__device__ __forceinline__ real2 mk2(real x, real y) { return make_float2(x, y); }
+#endif
 
 // even-odd folding of the symmetric GLL grids: HP mirrored node pairs of the
 // P-grid (plus its middle node when P is odd: HPE = ceil(P / 2) folded
@@ -56,6 +64,7 @@ typedef REAL real;
 constexpr int HP = P / 2;
 constexpr int HPE = (P + 1) / 2;
 constexpr int HQ = W;
+constexpr int FACE_ARR = 15;  // P x P arrays per face of the face phase's scratch
 // B1 is odd under the reflection of both grids, B0 and B2 even
 __host__ __device__ constexpr bool odd_mat(int m) { return m == 1; }
 // P x P matrices of the face phase: D and D^T are odd, MP and KP even
@@ -114,8 +123,9 @@ struct Tables {
   // pairs of folded entries for the packed FP32 contractions (two matrices
   // applied at once, see fwd_pm2): XE[0][i] = (FE[0][i], FE[0][i]),
   // XE[1][i] = (FE[0][i], FE[2][i]); XO likewise from FO
-  float2 XE[2][P * HPE];
-  float2 XO[2][P * HPE];
+  // (K = 2: (FE[1][i], FE[1][i]), used by general.cuh only)
+  real2 XE[3][P * HPE];
+  real2 XO[3][P * HPE];
 };
 __constant__ Tables c_tab;
 
@@ -342,15 +352,22 @@ __host__ __device__ constexpr bool packed_mode(int c, int mode) {
   return mode != hpse::MODE_TRANSPOSE || c != hpse::COEF_SCALAR;
 }
 
-__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+#if defined(HPSE_DOUBLE)
+__device__ __forceinline__ real2 fma2(real2 a, real2 b, real2 c) { return mk2(fma(a.x, b.x, c.x), fma(a.y, b.y, c.y)); }
+__device__ __forceinline__ real2 add2(real2 a, real2 b) { return mk2(a.x + b.x, a.y + b.y); }
+__device__ __forceinline__ real2 sub2(real2 a, real2 b) { return mk2(a.x - b.x, a.y - b.y); }
+#else
+__device__ __forceinline__ real2 fma2(real2 a, real2 b, real2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ real2 add2(real2 a, real2 b) { return __fadd2_rn(a, b); }
 // a - b, exactly rounded (a + (-1) b in one FMA)
-__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
-__device__ __forceinline__ float2 zero2() { return make_float2(0.f, 0.f); }
+__device__ __forceinline__ real2 sub2(real2 a, real2 b) { return __ffma2_rn(b, mk2(-1.f, -1.f), a); }
+#endif
+__device__ __forceinline__ real2 zero2() { return mk2(0, 0); }
 template <int H>
-__device__ __forceinline__ float half2_of(float2 v) { return H ? v.y : v.x; }
+__device__ __forceinline__ real half2_of(real2 v) { return H ? v.y : v.x; }
 
 // u[P] (pairs) -> e, o as fold_p, both halves at once
-__device__ __forceinline__ void fold_p2(const float2 *u, float2 *e, float2 *o) {
+__device__ __forceinline__ void fold_p2(const real2 *u, real2 *e, real2 *o) {
 #pragma unroll
   for (int j = 0; j < HP; ++j) {
     e[j] = add2(u[j], u[P - 1 - j]);
@@ -362,7 +379,7 @@ __device__ __forceinline__ void fold_p2(const float2 *u, float2 *e, float2 *o) {
   }
 }
 // v[Q] (pairs) -> ve, vo, vm as fold_q
-__device__ __forceinline__ void fold_q2(const float2 *v, float2 *ve, float2 *vo, float2 &vm) {
+__device__ __forceinline__ void fold_q2(const real2 *v, real2 *ve, real2 *vo, real2 &vm) {
 #pragma unroll
   for (int q = 0; q < HQ; ++q) {
     ve[q] = add2(v[q], v[Q - 1 - q]);
@@ -373,17 +390,17 @@ __device__ __forceinline__ void fold_q2(const float2 *v, float2 *ve, float2 *vo,
 
 // forward pair, output pair q: as fwd_pm for two even matrices
 template <int K>
-__device__ __forceinline__ void fwd_pm2(const float2 *e, const float2 *o, int q, float2 &pl, float2 &mi) {
+__device__ __forceinline__ void fwd_pm2(const real2 *e, const real2 *o, int q, real2 &pl, real2 &mi) {
 #pragma unroll
-  for (int j = 0; j < HPE; ++j) pl = __ffma2_rn(c_tab.XE[K][q * HPE + j], e[j], pl);
+  for (int j = 0; j < HPE; ++j) pl = fma2(c_tab.XE[K][q * HPE + j], e[j], pl);
   if (q < HQ) {
 #pragma unroll
-    for (int j = 0; j < HP; ++j) mi = __ffma2_rn(c_tab.XO[K][q * HPE + j], o[j], mi);
+    for (int j = 0; j < HP; ++j) mi = fma2(c_tab.XO[K][q * HPE + j], o[j], mi);
   }
 }
 // fwd_pm of matrix M on half H of a packed line
 template <int M, int H>
-__device__ __forceinline__ void fwd_pm_h(const float2 *e, const float2 *o, int q, real &pl, real &mi) {
+__device__ __forceinline__ void fwd_pm_h(const real2 *e, const real2 *o, int q, real &pl, real &mi) {
 #pragma unroll
   for (int j = 0; j < HPE; ++j) {
     if (!odd_mat(M)) pl += c_tab.FE[M][q * HPE + j] * half2_of<H>(e[j]);
@@ -397,32 +414,32 @@ __device__ __forceinline__ void fwd_pm_h(const float2 *e, const float2 *o, int q
 }
 // transpose pair: as rev_pair / rev_mid for two even matrices
 template <int K>
-__device__ __forceinline__ void rev_pair2(float2 ve, float2 vo, int q, float2 *pl, float2 *mi) {
+__device__ __forceinline__ void rev_pair2(real2 ve, real2 vo, int q, real2 *pl, real2 *mi) {
 #pragma unroll
   for (int k = 0; k < HPE; ++k) {
-    pl[k] = __ffma2_rn(c_tab.XE[K][q * HPE + k], ve, pl[k]);
-    if (k < HP) mi[k] = __ffma2_rn(c_tab.XO[K][q * HPE + k], vo, mi[k]);
+    pl[k] = fma2(c_tab.XE[K][q * HPE + k], ve, pl[k]);
+    if (k < HP) mi[k] = fma2(c_tab.XO[K][q * HPE + k], vo, mi[k]);
   }
 }
 template <int K>
-__device__ __forceinline__ void rev_mid2(float2 vm, float2 *pl) {
+__device__ __forceinline__ void rev_mid2(real2 vm, real2 *pl) {
 #pragma unroll
-  for (int k = 0; k < HPE; ++k) pl[k] = __ffma2_rn(c_tab.XE[K][HQ * HPE + k], vm, pl[k]);
+  for (int k = 0; k < HPE; ++k) pl[k] = fma2(c_tab.XE[K][HQ * HPE + k], vm, pl[k]);
 }
 // transpose of a whole folded pair of lines into output pair k: as rev_line
 template <int K>
-__device__ __forceinline__ void rev_line2(const float2 *ve, const float2 *vo, float2 vm, int k, float2 &pl,
-                                          float2 &mi) {
+__device__ __forceinline__ void rev_line2(const real2 *ve, const real2 *vo, real2 vm, int k, real2 &pl,
+                                          real2 &mi) {
 #pragma unroll
   for (int q = 0; q < HQ; ++q) {
-    pl = __ffma2_rn(c_tab.XE[K][q * HPE + k], ve[q], pl);
-    if (k < HP) mi = __ffma2_rn(c_tab.XO[K][q * HPE + k], vo[q], mi);
+    pl = fma2(c_tab.XE[K][q * HPE + k], ve[q], pl);
+    if (k < HP) mi = fma2(c_tab.XO[K][q * HPE + k], vo[q], mi);
   }
-  pl = __ffma2_rn(c_tab.XE[K][HQ * HPE + k], vm, pl);
+  pl = fma2(c_tab.XE[K][HQ * HPE + k], vm, pl);
 }
 // rev_line of matrix M on half H of a packed folded line
 template <int M, int H>
-__device__ __forceinline__ void rev_line_h(const float2 *ve, const float2 *vo, float2 vm, int k, real &pl,
+__device__ __forceinline__ void rev_line_h(const real2 *ve, const real2 *vo, real2 vm, int k, real &pl,
                                            real &mi) {
 #pragma unroll
   for (int q = 0; q < HQ; ++q) {
@@ -433,27 +450,30 @@ __device__ __forceinline__ void rev_line_h(const float2 *ve, const float2 *vo, f
   else if (k < HP) mi += c_tab.FO[M][HQ * HPE + k] * half2_of<H>(vm);
 }
 // store the pairs (q, Q-1-q) of two forward outputs: half .x to dx, .y to dy
-__device__ __forceinline__ void put_q2(real *dx, real *dy, int stride, int q, float2 pl, float2 mi) {
-  const float2 a = add2(pl, mi);
+__device__ __forceinline__ void put_q2(real *dx, real *dy, int stride, int q, real2 pl, real2 mi) {
+  const real2 a = add2(pl, mi);
   dx[q * stride] = a.x;
   dy[q * stride] = a.y;
   if (q < HQ) {
-    const float2 b = sub2(pl, mi);
+    const real2 b = sub2(pl, mi);
     dx[(Q - 1 - q) * stride] = b.x;
     dy[(Q - 1 - q) * stride] = b.y;
   }
 }
 // store the pairs (k, P-1-k) of two transposed outputs
-__device__ __forceinline__ void put_p2(real *dx, real *dy, int stride, int k, float2 pl, float2 mi) {
-  const float2 a = add2(pl, mi);
+__device__ __forceinline__ void put_p2(real *dx, real *dy, int stride, int k, real2 pl, real2 mi) {
+  const real2 a = add2(pl, mi);
   dx[k * stride] = a.x;
   dy[k * stride] = a.y;
   if (k < HP) {
-    const float2 b = sub2(pl, mi);
+    const real2 b = sub2(pl, mi);
     dx[(P - 1 - k) * stride] = b.x;
     dy[(P - 1 - k) * stride] = b.y;
   }
 }
+
+template <int COEF>
+struct TRows;  // ::S, the row stride of the T fields (defined with the face phase's sizes below)
 
 // x-stage: X0 = B0 u, X2 = B2 u (X1 = B1 u) along x for line l = (j, k)
 template <int COEF, int CI, int NC>
@@ -489,7 +509,7 @@ __device__ __forceinline__ void y_fwd_chunk(const real *e0, const real *o0, cons
     fwd_pm<0>(e2, o2, qb, pl2, ml2);
     if (var_coef(COEF)) fwd_pm<0>(e1, o1, qb, p10, m10);
     if (y_first(COEF)) fwd_pm<1>(e0, o0, qb, p01, m01);
-    const int o = k * Q2 + qa;  // + qb * Q
+    const int o = k * TRows<COEF>::S + qa;  // + qb * Q
     if (ok) {
       put_q(T00 + o, Q, qb, p00, m00);
       put_q(TL + o, Q, qb, sx2 * pl2 + sy2 * pl0, sx2 * ml2 + sy2 * ml0);
@@ -506,7 +526,7 @@ __device__ __forceinline__ void y_rev_chunk(const real *RZ, const real *R0, cons
                                             real *X0, real *X1, real *X2, int qa, int k, bool ok, real sx2,
                                             real sy2) {
   typedef Range<CI, NC, HPE> R;
-  const int o = k * Q2 + qa;  // + qb * Q
+  const int o = k * TRows<COEF>::S + qa;  // + qb * Q
   {
     real ze[HQ], zo[HQ], zm, re[HQ], ro[HQ], rm, ye[HQ], yo[HQ], ym;
     {
@@ -588,12 +608,12 @@ __device__ __forceinline__ void x_rev_chunk(const real *X0, const real *X1, cons
 // x-stage: e, o hold the folded line u in both halves: (B0 u, B2 u) packed,
 // B1 u (variable coefficient) scalar on the .x half
 template <int COEF, int CI, int NC>
-__device__ __forceinline__ void x_fwd_chunk2(const float2 *e, const float2 *o, real *X0, real *X1, real *X2, int l,
+__device__ __forceinline__ void x_fwd_chunk2(const real2 *e, const real2 *o, real *X0, real *X1, real *X2, int l,
                                              bool ok) {
   typedef Range<CI, NC, HQ + 1> R;
 #pragma unroll
   for (int q = R::B; q < R::E; ++q) {
-    float2 pl = zero2(), mi = zero2();
+    real2 pl = zero2(), mi = zero2();
     real p1 = 0, m1 = 0;
     fwd_pm2<1>(e, o, q, pl, mi);
     if (var_coef(COEF)) fwd_pm_h<1, 0>(e, o, q, p1, m1);
@@ -609,15 +629,15 @@ __device__ __forceinline__ void x_fwd_chunk2(const float2 *e, const float2 *o, r
 // w = (X2, X1) -> (B0 X2, B0 X1), B1 X0 scalar on d.x.  Laplacian:
 // w = (X0, X2) -> (B0 X0, B0 X2), B2 X0 scalar on w.x (d unused).
 template <int COEF, int CI, int NC>
-__device__ __forceinline__ void y_fwd_chunk2(const float2 *de, const float2 *dd, const float2 *we, const float2 *wo,
+__device__ __forceinline__ void y_fwd_chunk2(const real2 *de, const real2 *dd, const real2 *we, const real2 *wo,
                                              real *T00, real *TL, real *T10, real *T01, int qa, int k, bool ok,
                                              real sx2, real sy2) {
   typedef Range<CI, NC, HQ + 1> R;
 #pragma unroll
   for (int qb = R::B; qb < R::E; ++qb) {
-    const int o = k * Q2 + qa;  // + qb * Q
+    const int o = k * TRows<COEF>::S + qa;  // + qb * Q
     if (COEF == COEF_SCALAR) {
-      float2 ap = zero2(), am = zero2(), bp = zero2(), bm = zero2();
+      real2 ap = zero2(), am = zero2(), bp = zero2(), bm = zero2();
       real p01 = 0, m01 = 0;
       fwd_pm2<1>(de, dd, qb, ap, am);
       fwd_pm2<0>(we, wo, qb, bp, bm);
@@ -629,7 +649,7 @@ __device__ __forceinline__ void y_fwd_chunk2(const float2 *de, const float2 *dd,
         put_q(T01 + o, Q, qb, p01, m01);
       }
     } else {
-      float2 bp = zero2(), bm = zero2();
+      real2 bp = zero2(), bm = zero2();
       real pl0 = 0, ml0 = 0;
       fwd_pm2<0>(we, wo, qb, bp, bm);
       fwd_pm_h<2, 0>(we, wo, qb, pl0, ml0);
@@ -649,14 +669,14 @@ __device__ __forceinline__ void y_rev_chunk2(const real *RZ, const real *R0, con
                                              real *X0, real *X1, real *X2, int qa, int k, bool ok, real sx2,
                                              real sy2) {
   typedef Range<CI, NC, HPE> R;
-  const int o = k * Q2 + qa;  // + qb * Q
+  const int o = k * TRows<COEF>::S + qa;  // + qb * Q
   {
-    float2 ze[HQ], zo[HQ], zm;
+    real2 ze[HQ], zo[HQ], zm;
     real ye[HQ], yo[HQ], ym;
     {
-      float2 v[Q];
+      real2 v[Q];
 #pragma unroll
-      for (int qb = 0; qb < Q; ++qb) v[qb] = make_float2(RZ[o + qb * Q], R0[o + qb * Q]);
+      for (int qb = 0; qb < Q; ++qb) v[qb] = mk2(RZ[o + qb * Q], R0[o + qb * Q]);
       fold_q2(v, ze, zo, zm);
     }
     if (y_first(COEF)) {
@@ -667,7 +687,7 @@ __device__ __forceinline__ void y_rev_chunk2(const real *RZ, const real *R0, con
     }
 #pragma unroll
     for (int j = R::B; j < R::E; ++j) {
-      float2 pl = zero2(), mi = zero2();
+      real2 pl = zero2(), mi = zero2();
       real p2 = 0, m2 = 0, py = 0, my = 0;
       rev_line2<0>(ze, zo, zm, j, pl, mi);
       rev_line_h<2, 1>(ze, zo, zm, j, p2, m2);
@@ -702,12 +722,12 @@ template <int COEF, int CI, int NC>
 __device__ __forceinline__ void x_rev_chunk2(const real *X0, const real *X1, const real *X2, real *sy, int l,
                                              bool ok) {
   typedef Range<CI, NC, HPE> R;
-  float2 e[HQ], o[HQ], m;
+  real2 e[HQ], o[HQ], m;
   real e1[HQ], o1[HQ], m1v;
   {
-    float2 v[Q];
+    real2 v[Q];
 #pragma unroll
-    for (int q = 0; q < Q; ++q) v[q] = make_float2(X0[l * Q + q], X2[l * Q + q]);
+    for (int q = 0; q < Q; ++q) v[q] = mk2(X0[l * Q + q], X2[l * Q + q]);
     fold_q2(v, e, o, m);
   }
   if (var_coef(COEF)) {
@@ -718,7 +738,7 @@ __device__ __forceinline__ void x_rev_chunk2(const real *X0, const real *X1, con
   }
 #pragma unroll
   for (int i = R::B; i < R::E; ++i) {
-    float2 pl = zero2(), mi = zero2();
+    real2 pl = zero2(), mi = zero2();
     real p1 = 0, q1 = 0;
     rev_line2<1>(e, o, m, i, pl, mi);
     if (var_coef(COEF)) rev_line<1>(e1, o1, m1v, i, p1, q1);
@@ -748,8 +768,6 @@ __device__ __forceinline__ void x_rev_chunk2(const real *X0, const real *X1, con
 // Scratch per face: 14 arrays of P x P (the G_k of the norm products reuse
 // the J slots, the transposed tangential derivatives the A slots).
 // ---------------------------------------------------------------------------
-constexpr int FACE_ARR = 15;
-
 template <int MODE>
 __device__ __forceinline__ real nb_value(const ApplyArgs &A, int64_t idx, real bt) {
   if (MODE == MODE_PCG) return A.z[idx] + bt * A.u[idx];
@@ -813,6 +831,35 @@ __device__ __forceinline__ FaceMeta *face_meta(real *stab) {
   const uintptr_t p = reinterpret_cast<uintptr_t>(stab + P2);
   return reinterpret_cast<FaceMeta *>((p + 7) & ~(uintptr_t)7);
 }
+// Row stride of T fields of P rows of Q^2 values (the y-stage's output per
+// k-plane).  A warp of the y-stages holds lines (qa, k) with qa fastest: Q lanes
+// of one plane, the next lanes of the following one.  With stride Q^2 those runs
+// overlap in the 32 banks (W = 8: Q^2 = 289 = 1 mod 32, two-way conflicts on
+// every T access of both y-stages, a third of the FP32 kernel's shared
+// wavefronts); FP32 rows are padded to a stride of Q mod 32, which makes a
+// warp's addresses distinct, where the padding costs no resident CTA
+// (config 2's apply 418 -> 410 us at 16 rhs, W = 7 306 -> 288 us).
+constexpr int T_PAD = sizeof(real) == 4 ? (((Q - Q2) % 32) + 32) % 32 : 0;
+// dynamic shared memory of an apply CTA: su | NX X fields | T region | D, face data | reduction
+constexpr size_t apply_bytes(int nx, int ntf, int ts) {
+  const int t = ntf * ts * P, need = P3 + 6 * FACE_ARR * P2;
+  const size_t tot = (size_t)(P3 + nx * QP2 + (t > need ? t : need) + P2 + FACE_META_REALS);
+  return ((tot * sizeof(real) + 15) / 16) * 16 + 64 * sizeof(double);
+}
+constexpr int sm_ctas(size_t bytes, int most) {
+  const int n = (int)(233472 / (bytes + 1024));
+  return n < most ? n : most;
+}
+constexpr int t_stride(int nx, int ntf, int minb) {
+  return sm_ctas(apply_bytes(nx, ntf, Q2 + T_PAD), minb) == sm_ctas(apply_bytes(nx, ntf, Q2), minb) ? Q2 + T_PAD : Q2;
+}
+template <int COEF>
+struct TRows {
+  static constexpr int NX = var_coef(COEF) ? 3 : 2;
+  static constexpr int NTF = y_first(COEF) ? 4 : (var_coef(COEF) ? 3 : 2);
+  static constexpr int S = t_stride(NX, NTF, APPLY_MINB);
+};
+
 template <int COEF, int MODE>
 __device__ __forceinline__ void face_meta_fill(const ApplyArgs &A, int e, int r, const real *geo_e, FaceMeta *M,
                                                int f) {
@@ -1163,10 +1210,11 @@ struct ColumnRho<true> {
 };
 
 // rho[q] of one z-column in place, in the column's own slots of the T
-// fields (q -> T00 / TL row q mod P; Q <= 2P): the forward holds the
+// fields (q -> row q of T00 and TL, which follow one another; Q <= 2P): the forward holds the
 // column's T inputs in registers before it writes rho, the transpose stores
 // its outputs there after its last read of rho.  Lanes past the last column
 // read the last column's rho and write nothing.
+template <int S>
 struct ColumnRhoT {
   real *p;
   bool w;
@@ -1183,7 +1231,7 @@ struct ColumnRhoT {
     p = T + col;
     w = ok;
   }
-  __device__ __forceinline__ Ref operator[](int q) { return Ref{p + (q / P) * Q2P + (q % P) * Q2, w}; }
+  __device__ __forceinline__ Ref operator[](int q) { return Ref{p + q * S, w}; }
 };
 
 // warp-uniform dispatch of a runtime chunk index to its compile-time instance
@@ -1203,25 +1251,29 @@ struct ColumnRhoT {
 // ---------------------------------------------------------------------------
 template <int COEF>
 struct ApplyLayout {
-  static constexpr int NX = (var_coef(COEF)) ? 3 : 2;
-  static constexpr int NTF = y_first(COEF) ? 4 : (var_coef(COEF) ? 3 : 2);
-  static constexpr int T_REGION0 = NTF * Q2P;
+  static constexpr int NX = TRows<COEF>::NX;
+  static constexpr int NTF = TRows<COEF>::NTF;
+  static constexpr int TS = TRows<COEF>::S;  // row stride of the T fields
+  static constexpr int T_REGION0 = NTF * TS * P;
   static constexpr int T_NEED = P3 + 6 * FACE_ARR * P2;
   static constexpr int T_REGION = T_REGION0 > T_NEED ? T_REGION0 : T_NEED;
   static constexpr int TABS = P2 + FACE_META_REALS;  // D copy, then the face phase's per-face data
   static constexpr int TOTAL0 = P3 + NX * QP2 + T_REGION + TABS;
   // the z-stage's pointwise residual rho per column in shared memory (Q
   // entries per column, one spare column for the lanes past the last one)
-  // where that keeps APPLY_MINB CTAs per SM; else in registers
+  // where that keeps APPLY_MINB CTAs per SM
   static constexpr int RHO_LEN = Q * (Q2 + 1);
-  // packed z-stage: rho in place in the T fields (ColumnRhoT), no buffer
-  static constexpr bool RHO_INPLACE = packed_coef(COEF, 4) || packed_coef(COEF, 8);
+  // rho in place in the T fields (ColumnRhoT), no buffer: FP32 (a batch of edge
+  // neighbourhoods of degree 2 to 8: 319 -> 252 us, its 676 bytes of spills
+  // gone), and FP64 where the buffer does not fit (W = 10: 2.91 -> 2.78 ms);
+  // below, FP64 is up to 4 % faster with the buffer
+  static constexpr bool RHO_FITS =
+      ((size_t)(TOTAL0 + RHO_LEN) * sizeof(real) + 64 * sizeof(double) + 1024) * APPLY_MINB <= 232448;
+  static constexpr bool RHO_INPLACE = sizeof(real) == 4 || !RHO_FITS;
 #if defined(HPSE_APPLY_RHO_REG)
   static constexpr bool RHO_SMEM = false;  // set at build time (layout experiments)
 #else
-  static constexpr bool RHO_SMEM =
-      !RHO_INPLACE &&
-      (((size_t)(TOTAL0 + RHO_LEN) * sizeof(real) + 64 * sizeof(double) + 1024) * APPLY_MINB <= 232448);
+  static constexpr bool RHO_SMEM = !RHO_INPLACE && RHO_FITS;
 #endif
   static constexpr int TOTAL = TOTAL0 + (RHO_SMEM ? RHO_LEN : 0);
   // the FP64 reduction buffer starts on a 16-byte boundary whatever REAL is
@@ -1241,7 +1293,8 @@ __global__ void __launch_bounds__(NT, APPLY_MINB) k_apply(const ApplyArgs A) {
   double *red = reinterpret_cast<double *>(smem_raw + L::RED_OFF);
   static_assert(L::RED_OFF % 16 == 0, "reduction buffer must be 16-byte aligned");
   real *X0 = sX, *X2 = sX + QP2, *X1 = sX + 2 * QP2;
-  real *T00 = sT, *TL = sT + Q2P, *T10 = sT + 2 * Q2P, *T01 = sT + 3 * Q2P;
+  constexpr int TS = L::TS, TF = TS * P;
+  real *T00 = sT, *TL = sT + TF, *T10 = sT + 2 * TF, *T01 = sT + 3 * TF;
 
   const int item = blockIdx.x;
   const int ge = item / A.n_rhs;
@@ -1285,11 +1338,11 @@ __global__ void __launch_bounds__(NT, APPLY_MINB) k_apply(const ApplyArgs A) {
           fold_p(v, e, o);
         }
         if constexpr (packed_coef(COEF, 1)) {
-          float2 e2[HPE], o2[HPE];
+          real2 e2[HPE], o2[HPE];
 #pragma unroll
           for (int j = 0; j < HPE; ++j) {
-            e2[j] = make_float2(e[j], e[j]);
-            o2[j] = make_float2(o[j], o[j]);
+            e2[j] = mk2(e[j], e[j]);
+            o2[j] = mk2(o[j], o[j]);
           }
 #define XF_CALL(CI) x_fwd_chunk2<COEF, (CI < LS::NC ? CI : 0), LS::NC>(e2, o2, X0, X1, X2, l, ok)
           HPSE_DISPATCH4(LS::NC, c, XF_CALL);
@@ -1312,22 +1365,22 @@ __global__ void __launch_bounds__(NT, APPLY_MINB) k_apply(const ApplyArgs A) {
         const int l = ok ? lp : QP - 1;
         const int qa = l % Q, k = l / Q;
         if constexpr (packed_coef(COEF, 2)) {
-          float2 de[HPE], dd[HPE], we[HPE], wo[HPE];
+          real2 de[HPE], dd[HPE], we[HPE], wo[HPE];
           {
-            float2 v[P];
+            real2 v[P];
             if (COEF == COEF_SCALAR) {
 #pragma unroll
               for (int j = 0; j < P; ++j) {
                 const real x0 = X0[(k * P + j) * Q + qa];
-                v[j] = make_float2(x0, x0);
+                v[j] = mk2(x0, x0);
               }
               fold_p2(v, de, dd);
 #pragma unroll
-              for (int j = 0; j < P; ++j) v[j] = make_float2(X2[(k * P + j) * Q + qa], X1[(k * P + j) * Q + qa]);
+              for (int j = 0; j < P; ++j) v[j] = mk2(X2[(k * P + j) * Q + qa], X1[(k * P + j) * Q + qa]);
               fold_p2(v, we, wo);
             } else {
 #pragma unroll
-              for (int j = 0; j < P; ++j) v[j] = make_float2(X0[(k * P + j) * Q + qa], X2[(k * P + j) * Q + qa]);
+              for (int j = 0; j < P; ++j) v[j] = mk2(X0[(k * P + j) * Q + qa], X2[(k * P + j) * Q + qa]);
               fold_p2(v, we, wo);
             }
           }
@@ -1380,7 +1433,7 @@ __global__ void __launch_bounds__(NT, APPLY_MINB) k_apply(const ApplyArgs A) {
         (COEF == COEF_EDGE || COEF == COEF_VERTEX_EDGE) ? sz2 * A.kappa[(int64_t)e * hpse::KAPPA_STRIDE + qa] : sz2;
     // lanes past the last column keep their rho in the spare column Q2
     constexpr bool inplace = L::RHO_INPLACE && packed_mode(COEF, MODE);
-    std::conditional_t<inplace, ColumnRhoT, ColumnRho<L::RHO_SMEM>> rho;
+    std::conditional_t<inplace, ColumnRhoT<TS>, ColumnRho<L::RHO_SMEM>> rho;
     if constexpr (inplace) rho.bind(sT, l, ok);
     else rho.bind(srho, ok ? l : Q2);
     if (MODE == MODE_TRANSPOSE) {
@@ -1390,26 +1443,26 @@ __global__ void __launch_bounds__(NT, APPLY_MINB) k_apply(const ApplyArgs A) {
       // -div(a grad u): A = (TL, T10) -> (p0, px) = (B0 TL, B0 T10),
       // B = (T01, T00) -> (py, p2) = (B0 T01, B2 T00), p1 = B1 T00 on B.y;
       // Laplacian: B = (TL, T00) -> (p0, p2)
-      float2 eA[HPE], oA[HPE], eB[HPE], oB[HPE];
+      real2 eA[HPE], oA[HPE], eB[HPE], oB[HPE];
       {
-        float2 v[P];
+        real2 v[P];
         if (COEF == COEF_SCALAR) {
 #pragma unroll
-          for (int k = 0; k < P; ++k) v[k] = make_float2(TL[k * Q2 + l], T10[k * Q2 + l]);
+          for (int k = 0; k < P; ++k) v[k] = mk2(TL[k * TS + l], T10[k * TS + l]);
           fold_p2(v, eA, oA);
 #pragma unroll
-          for (int k = 0; k < P; ++k) v[k] = make_float2(T01[k * Q2 + l], T00[k * Q2 + l]);
+          for (int k = 0; k < P; ++k) v[k] = mk2(T01[k * TS + l], T00[k * TS + l]);
           fold_p2(v, eB, oB);
         } else {
 #pragma unroll
-          for (int k = 0; k < P; ++k) v[k] = make_float2(TL[k * Q2 + l], T00[k * Q2 + l]);
+          for (int k = 0; k < P; ++k) v[k] = mk2(TL[k * TS + l], T00[k * TS + l]);
           fold_p2(v, eB, oB);
         }
       }
       const real wab = c_tab.WQ[qa] * c_tab.WQ[qb] * Jac;
 #pragma unroll
       for (int qc = 0; qc <= HQ; ++qc) {
-        float2 ap = zero2(), am = zero2(), bp = zero2(), bm = zero2();
+        real2 ap = zero2(), am = zero2(), bp = zero2(), bm = zero2();
         real p1 = 0, m1 = 0;
         fwd_pm2<1>(eB, oB, qc, bp, bm);
         if (COEF == COEF_SCALAR) {
@@ -1420,9 +1473,9 @@ __global__ void __launch_bounds__(NT, APPLY_MINB) k_apply(const ApplyArgs A) {
         for (int side = 0; side < (qc < HQ ? 2 : 1); ++side) {
           const int q = side ? Q - 1 - qc : qc;
           const real sg = side ? (real)-1 : (real)1;
-          const float2 b = side ? sub2(bp, bm) : add2(bp, bm);
+          const real2 b = side ? sub2(bp, bm) : add2(bp, bm);
           if (COEF == COEF_SCALAR) {
-            const float2 a = side ? sub2(ap, am) : add2(ap, am);
+            const real2 a = side ? sub2(ap, am) : add2(ap, am);
             const real sigma0 = sz2c * b.y + a.x;
             real mq, dx, dy, dz;
             load_coef4(A.coef + 4 * (cbase + (int64_t)q * Q2), mq, dx, dy, dz);
@@ -1438,19 +1491,19 @@ __global__ void __launch_bounds__(NT, APPLY_MINB) k_apply(const ApplyArgs A) {
       {
         real v[P];
 #pragma unroll
-        for (int k = 0; k < P; ++k) v[k] = T00[k * Q2 + l];
+        for (int k = 0; k < P; ++k) v[k] = T00[k * TS + l];
         fold_p(v, e00, o00);
 #pragma unroll
-        for (int k = 0; k < P; ++k) v[k] = TL[k * Q2 + l];
+        for (int k = 0; k < P; ++k) v[k] = TL[k * TS + l];
         fold_p(v, eL, oL);
         if (var_coef(COEF)) {
 #pragma unroll
-          for (int k = 0; k < P; ++k) v[k] = T10[k * Q2 + l];
+          for (int k = 0; k < P; ++k) v[k] = T10[k * TS + l];
           fold_p(v, e10, o10);
         }
         if (y_first(COEF)) {
 #pragma unroll
-          for (int k = 0; k < P; ++k) v[k] = T01[k * Q2 + l];
+          for (int k = 0; k < P; ++k) v[k] = T01[k * TS + l];
           fold_p(v, e01, o01);
         }
       }
@@ -1487,12 +1540,12 @@ __global__ void __launch_bounds__(NT, APPLY_MINB) k_apply(const ApplyArgs A) {
       // -div(a grad u): (rho, d_x rho) -> (rp, xp) by (B0, B0), (d_y rho,
       // sz2 rho) -> (yp, zp) by (B0, B2), d_z rho by B1 into zp (scalar);
       // Laplacian: (rho, sz2 rho) -> (rp, zp) by (B0, B2)
-      float2 pa[HPE], ma[HPE], pb[HPE], mb[HPE];
+      real2 pa[HPE], ma[HPE], pb[HPE], mb[HPE];
 #pragma unroll
       for (int k = 0; k < HPE; ++k) pa[k] = ma[k] = pb[k] = mb[k] = zero2();
 #pragma unroll
       for (int qc = 0; qc <= HQ; ++qc) {
-        float2 va[2], vb[2];
+        real2 va[2], vb[2];
         real sd[2];
 #pragma unroll
         for (int side = 0; side < (qc < HQ ? 2 : 1); ++side) {
@@ -1501,11 +1554,11 @@ __global__ void __launch_bounds__(NT, APPLY_MINB) k_apply(const ApplyArgs A) {
           if (COEF == COEF_SCALAR) {
             real mq, dx, dy, dz;
             load_coef4(A.coef + 4 * (cbase + (int64_t)q * Q2), mq, dx, dy, dz);
-            va[side] = make_float2(rq, dx * rq);
-            vb[side] = make_float2(dy * rq, sz2c * rq);
+            va[side] = mk2(rq, dx * rq);
+            vb[side] = mk2(dy * rq, sz2c * rq);
             sd[side] = dz * rq;
           } else {
-            vb[side] = make_float2(rq, sz2c * rq);
+            vb[side] = mk2(rq, sz2c * rq);
           }
         }
         if (qc < HQ) {
@@ -1532,10 +1585,10 @@ __global__ void __launch_bounds__(NT, APPLY_MINB) k_apply(const ApplyArgs A) {
 #pragma unroll
         for (int k = 0; k < HPE; ++k) {
           if (COEF == COEF_SCALAR) {
-            put_p2(TL + l, T10 + l, Q2, k, pa[k], ma[k]);
-            put_p2(T01 + l, T00 + l, Q2, k, pb[k], mb[k]);
+            put_p2(TL + l, T10 + l, TS, k, pa[k], ma[k]);
+            put_p2(T01 + l, T00 + l, TS, k, pb[k], mb[k]);
           } else {
-            put_p2(TL + l, T00 + l, Q2, k, pb[k], mb[k]);
+            put_p2(TL + l, T00 + l, TS, k, pb[k], mb[k]);
           }
         }
       }
@@ -1588,10 +1641,10 @@ __global__ void __launch_bounds__(NT, APPLY_MINB) k_apply(const ApplyArgs A) {
       if (ok) {
 #pragma unroll
         for (int k = 0; k < HPE; ++k) {
-          put_p(T00 + l, Q2, k, zp[k], zm[k]);
-          put_p(TL + l, Q2, k, rp[k], rm[k]);
-          if (var_coef(COEF)) put_p(T10 + l, Q2, k, xp[k], xm[k]);
-          if (y_first(COEF)) put_p(T01 + l, Q2, k, yp[k], ym[k]);
+          put_p(T00 + l, TS, k, zp[k], zm[k]);
+          put_p(TL + l, TS, k, rp[k], rm[k]);
+          if (var_coef(COEF)) put_p(T10 + l, TS, k, xp[k], xm[k]);
+          if (y_first(COEF)) put_p(T01 + l, TS, k, yp[k], ym[k]);
         }
       }
     }
