@@ -420,9 +420,8 @@ hpse_status hpse_conforming_correction(hpse_mesh *m, const double *u, double *p,
  *                         data term (the backward of the residual map); z and
  *                         y device, of precision prec.
  * prec: HPSE_FP64, or HPSE_FP32 (the sum factorisations in FP32 with the FP64
- * tables and data rounded to FP32).  Asynchronous on `stream`.  Both use a
- * scratch buffer the handle allocates on first use.  HPSE_ERR_INVALID_ARG for
- * neighbourhood meshes, bad pointers or prec; HPSE_ERR_NO_DATA before
+ * tables and data rounded to FP32).  Asynchronous on `stream`.
+ * HPSE_ERR_INVALID_ARG for neighbourhood meshes, bad pointers or prec; HPSE_ERR_NO_DATA before
  * hpse_set_data. */
 hpse_status hpse_apply_residual(hpse_mesh *m, int32_t prec, const void *u, void *z, void *stream);
 hpse_status hpse_apply_transpose(hpse_mesh *m, int32_t prec, const void *z, void *y, void *stream);

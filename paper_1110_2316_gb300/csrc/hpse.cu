@@ -213,14 +213,14 @@ struct hpse_mesh {
   std::vector<Group> groups;
   // device mesh arrays
   // d_prob: problem of each vector item (n_elem + n_corner entries)
-  DevBuf d_dof_off, d_nbr, d_geo64, d_geo32, d_prob, d_coef_off, d_prob_ptr, d_prob_elems, d_elem_W;
+  DevBuf d_dof_off, d_nbr, d_geo64, d_geo32, d_sqj64, d_sqj32, d_prob, d_coef_off, d_prob_ptr, d_prob_elems, d_elem_W;
   DevBuf d_coef64, d_coef32;  // [nquad][4] (m, d_x, d_y, d_z) per point (COEF_SCALAR);
                               // [nquad][12] (w J, C_11 .. C_0, 0) (HPSE_COEF_GENERAL)
   DevBuf d_b;                 // FP64 right-hand side
   DevBuf d_f;                 // FP64 source at the volume points [n_rhs][nquad]
   DevBuf d_aux;               // FP64 [5][nquad]: w J, a, a_x, a_y, a_z at the volume points
   DevBuf d_tabs_ptr;          // device array of the per-degree FP64 table pointers
-  DevBuf d_scr_fields, d_scr_rho;  // scratch of the residual map and its transpose
+  DevBuf d_scr_rho;           // scratch of the integration-by-parts transpose
   // conforming correction (box meshes; built on first use): per element corner
   // (8) and edge (12) the shared vertex / edge, their members (CSR) and
   // Dirichlet flags, the linear blends (1 -+ x)/2 at the GLL nodes per degree
@@ -1059,7 +1059,7 @@ static hpse_status launch_apply_all(hpse_mesh *m, int mode, ApplyArgsT<T> base_a
     ++g_launches;
   }
   CK(group_join(m, s));
-  if (m->has_mixed && mode != MODE_TRANSPOSE && !base_args.skip_faces) {
+  if (m->has_mixed && mode != MODE_TRANSPOSE && mode != MODE_RESIDUAL && !base_args.skip_faces) {
     // faces between unequal degrees, after every element's apply (PCG mode:
     // the new search direction of every element is in pnew by then)
     const T *uu = mode == MODE_PCG ? base_args.pnew : base_args.u;
@@ -1067,7 +1067,7 @@ static hpse_status launch_apply_all(hpse_mesh *m, int mode, ApplyArgsT<T> base_a
                                      base_args.self_only, 0, s);
     if (st != HPSE_OK) return st;
   }
-  if (m->curved && mode != MODE_TRANSPOSE && !base_args.skip_faces) {
+  if (m->curved && mode != MODE_TRANSPOSE && mode != MODE_RESIDUAL && !base_args.skip_faces) {
     const T *uu = mode == MODE_PCG ? base_args.pnew : base_args.u;
     hpse_status st = launch_curved<T>(m, mode, uu, base_args.y, base_args.partial, base_args.n_rhs,
                                       base_args.self_only, 0, s);
@@ -2252,7 +2252,8 @@ extern "C" hpse_status hpse_setup_mesh(const hpse_mesh_desc *d, int device, hpse
     }
   }
   std::vector<double> geo(4 * (size_t)E);
-  std::vector<float> geo32(4 * (size_t)E);
+  std::vector<float> geo32(4 * (size_t)E), sqj32(E);
+  std::vector<double> sqj(E);  // square roots of the Jacobians (residual map)
   for (int e = 0; e < E; ++e) {
     double J = 1.0;
     for (int a = 0; a < 3; ++a) {
@@ -2262,6 +2263,8 @@ extern "C" hpse_status hpse_setup_mesh(const hpse_mesh_desc *d, int device, hpse
     }
     geo[4 * e + 3] = J;
     for (int k = 0; k < 4; ++k) geo32[4 * e + k] = (float)geo[4 * e + k];
+    sqj[e] = std::sqrt(geo[4 * e + 3]);
+    sqj32[e] = (float)sqj[e];
   }
   if (nbhd) {
     hpse_status st = setup_edge(m.get());
@@ -2273,6 +2276,8 @@ extern "C" hpse_status hpse_setup_mesh(const hpse_mesh_desc *d, int device, hpse
   CK(upload(m->d_nbr, m->nbr));
   CK(upload(m->d_geo64, geo));
   CK(upload(m->d_geo32, geo32));
+  CK(upload(m->d_sqj64, sqj));
+  CK(upload(m->d_sqj32, sqj32));
   if (m->has_nr || m->has_mixed || m->curved) {
     std::vector<float> g32(m->fgam.begin(), m->fgam.end());
     CK(upload(m->d_fbc, m->fbc));
@@ -3989,22 +3994,6 @@ __global__ void k_fields_T(FieldArgs A, const double *wf) {
   for (int t = threadIdx.x; t < P * P * P; t += nt) A.out[base + t] = Y[t];
 }
 
-// residual map at the points: z = sqrt(wJ) (L u - f)
-template <typename T>
-__global__ void k_resid_points(int64_t nquad, int n_rhs, const double *aux, const double *f, const T *fields,
-                               T *z) {
-  const int64_t n = nquad * n_rhs;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t r = i / nquad, q = i - r * nquad;
-    const T *fl = fields + r * 5 * nquad;
-    const T wJ = (T)aux[q], a = (T)aux[nquad + q];
-    const T Lu = -a * fl[4 * nquad + q] -
-                 ((T)aux[2 * nquad + q] * fl[nquad + q] + (T)aux[3 * nquad + q] * fl[2 * nquad + q] +
-                  (T)aux[4 * nquad + q] * fl[3 * nquad + q]);
-    z[i] = sqrt(wJ) * (Lu - (T)f[i]);
-  }
-}
-
 // rho = -sqrt(wJ) a z: the weights of S^T z in the sum-factorised transpose kernel
 template <typename T>
 __global__ void k_rho_from_z(int64_t nquad, int n_rhs, const double *aux, const T *z, double *rho) {
@@ -4166,25 +4155,19 @@ extern "C" hpse_status hpse_quad_weights(hpse_mesh *m, double *out, void *stream
   return HPSE_OK;
 }
 
-static hpse_status ensure_scratch(hpse_mesh *m, size_t fbytes) {
-  const size_t nf = (size_t)5 * m->n_rhs * m->nquad * fbytes;
-  const size_t nr = (size_t)m->n_rhs * m->nquad * sizeof(double);
-  if (m->d_scr_fields.bytes < nf) CK(m->d_scr_fields.alloc(nf));
-  if (m->d_scr_rho.bytes != nr) CK(m->d_scr_rho.alloc(nr));
-  return HPSE_OK;
-}
-
+// the residual map in the operator kernels (MODE_RESIDUAL): the z-stage writes
+// z at the points, so no point field goes through memory.  (The five point
+// fields and a second pass took 491 + 54 us of the 881 us of a map and its
+// transpose over 512 elements of degree 4 to 10.)
 template <typename T>
 static hpse_status residual_t(hpse_mesh *m, const T *u, T *z, cudaStream_t s) {
-  hpse_status st = ensure_scratch(m, sizeof(T));
-  if (st != HPSE_OK) return st;
-  st = launch_fields<T>(m, u, (T *)m->d_scr_fields.p, s);
-  if (st != HPSE_OK) return st;
-  k_resid_points<T><<<1024, 256, 0, s>>>(m->nquad, m->n_rhs, m->d_aux.as<double>(), m->d_f.as<double>(),
-                                         (const T *)m->d_scr_fields.p, z);
-  CK(cudaGetLastError());
-  ++g_launches;
-  return HPSE_OK;
+  ApplyArgsT<T> a = apply_args<T>(m, m->groups[0], u, nullptr);
+  a.aux = m->d_aux.as<double>();
+  a.sqj = (sizeof(T) == 8) ? (const T *)m->d_sqj64.p : (const T *)m->d_sqj32.p;
+  a.f = m->d_f.as<double>();
+  a.zout = z;
+  a.skip_faces = 1;
+  return launch_apply_all<T>(m, MODE_RESIDUAL, a, s);
 }
 
 extern "C" hpse_status hpse_apply_residual(hpse_mesh *m, int32_t prec, const void *u, void *z, void *stream) {
@@ -4202,13 +4185,10 @@ extern "C" hpse_status hpse_apply_residual(hpse_mesh *m, int32_t prec, const voi
 
 template <typename T>
 static hpse_status transpose_t(hpse_mesh *m, const T *z, T *y, cudaStream_t s) {
-  hpse_status st = ensure_scratch(m, sizeof(double));
-  if (st != HPSE_OK) return st;
-  k_rho_from_z<T><<<1024, 256, 0, s>>>(m->nquad, m->n_rhs, m->d_aux.as<double>(), z, m->d_scr_rho.as<double>());
-  CK(cudaGetLastError());
-  ++g_launches;
   ApplyArgsT<T> a = apply_args<T>(m, m->groups[0], nullptr, y);
-  a.rho = m->d_scr_rho.as<double>();
+  a.aux = m->d_aux.as<double>();
+  a.sqj = (sizeof(T) == 8) ? (const T *)m->d_sqj64.p : (const T *)m->d_sqj32.p;
+  a.zin = z;
   a.skip_faces = 1;
   return launch_apply_all<T>(m, MODE_TRANSPOSE, a, s);
 }
@@ -4229,8 +4209,8 @@ extern "C" hpse_status hpse_apply_transpose(hpse_mesh *m, int32_t prec, const vo
 // the volume transpose in integration-by-parts form (eq. 5.45-5.48), per degree group
 template <typename T>
 static hpse_status transpose_ibp_t(hpse_mesh *m, const T *z, T *y, cudaStream_t s) {
-  hpse_status st = ensure_scratch(m, sizeof(double));
-  if (st != HPSE_OK) return st;
+  const size_t nr = (size_t)m->n_rhs * m->nquad * sizeof(double);
+  if (m->d_scr_rho.bytes != nr) CK(m->d_scr_rho.alloc(nr));
   k_rho_from_z<T><<<1024, 256, 0, s>>>(m->nquad, m->n_rhs, m->d_aux.as<double>(), z, m->d_scr_rho.as<double>());
   CK(cudaGetLastError());
   ++g_launches;

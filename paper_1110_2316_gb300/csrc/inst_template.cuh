@@ -1,6 +1,7 @@
 // inst_template.cuh -- launchers for one (REAL, WDEG) instantiation of
 // kernels.cuh.  A generated translation unit defines REAL, WDEG,
 // HPSE_REGISTER_NAME (and HPSE_DOUBLE for REAL = double), then includes this.
+#include <cmath>
 #include <vector>
 
 #include "kernels.cuh"
@@ -22,10 +23,12 @@ cudaError_t apply_fn(int coef, int mode, const void *args, int n_items, int thre
     if (mode == MODE_PLAIN) return launch_apply_t<COEF_LAPLACE, MODE_PLAIN>(args, n_items, threads, s);
     if (mode == MODE_PCG) return launch_apply_t<COEF_LAPLACE, MODE_PCG>(args, n_items, threads, s);
     if (mode == MODE_TRANSPOSE) return launch_apply_t<COEF_LAPLACE, MODE_TRANSPOSE>(args, n_items, threads, s);
+    if (mode == MODE_RESIDUAL) return launch_apply_t<COEF_LAPLACE, MODE_RESIDUAL>(args, n_items, threads, s);
   } else if (coef == COEF_SCALAR) {
     if (mode == MODE_PLAIN) return launch_apply_t<COEF_SCALAR, MODE_PLAIN>(args, n_items, threads, s);
     if (mode == MODE_PCG) return launch_apply_t<COEF_SCALAR, MODE_PCG>(args, n_items, threads, s);
     if (mode == MODE_TRANSPOSE) return launch_apply_t<COEF_SCALAR, MODE_TRANSPOSE>(args, n_items, threads, s);
+    if (mode == MODE_RESIDUAL) return launch_apply_t<COEF_SCALAR, MODE_RESIDUAL>(args, n_items, threads, s);
   } else if (coef == COEF_EDGE) {
     if (mode == MODE_PLAIN) return launch_apply_t<COEF_EDGE, MODE_PLAIN>(args, n_items, threads, s);
     if (mode == MODE_PCG) return launch_apply_t<COEF_EDGE, MODE_PCG>(args, n_items, threads, s);
@@ -156,6 +159,7 @@ cudaError_t upload_fn(const double *pk) {
         t.PF[m][0][i * HPE + j] = (real)(mid ? x(i, j) : 0.5 * (x(i, j) + x(i, P - 1 - j)));
         t.PF[m][1][i * HPE + j] = (real)(mid ? 0.0 : 0.5 * (x(i, j) - x(i, P - 1 - j)));
       }
+  for (int i = 0; i < Q; ++i) t.SQ[i] = (real)std::sqrt(pk[o + i]);
   for (int i = 0; i < Q; ++i) t.WQ[i] = (real)pk[o++];
   for (int i = 0; i < P; ++i) t.MU[i] = (real)pk[o++];
   cudaError_t err = cudaMemcpyToSymbol(c_tab, &t, sizeof(Tables));
@@ -179,9 +183,11 @@ cudaError_t upload_fn(const double *pk) {
   if ((e2 = set_smem_attr<COEF_LAPLACE, MODE_PLAIN>()) != cudaSuccess) return e2;
   if ((e2 = set_smem_attr<COEF_LAPLACE, MODE_PCG>()) != cudaSuccess) return e2;
   if ((e2 = set_smem_attr<COEF_LAPLACE, MODE_TRANSPOSE>()) != cudaSuccess) return e2;
+  if ((e2 = set_smem_attr<COEF_LAPLACE, MODE_RESIDUAL>()) != cudaSuccess) return e2;
   if ((e2 = set_smem_attr<COEF_SCALAR, MODE_PLAIN>()) != cudaSuccess) return e2;
   if ((e2 = set_smem_attr<COEF_SCALAR, MODE_PCG>()) != cudaSuccess) return e2;
   if ((e2 = set_smem_attr<COEF_SCALAR, MODE_TRANSPOSE>()) != cudaSuccess) return e2;
+  if ((e2 = set_smem_attr<COEF_SCALAR, MODE_RESIDUAL>()) != cudaSuccess) return e2;
   if ((e2 = set_smem_attr<COEF_EDGE, MODE_PLAIN>()) != cudaSuccess) return e2;
   if ((e2 = set_smem_attr<COEF_EDGE, MODE_PCG>()) != cudaSuccess) return e2;
   if ((e2 = set_smem_attr<COEF_EDGE, MODE_TRANSPOSE>()) != cudaSuccess) return e2;

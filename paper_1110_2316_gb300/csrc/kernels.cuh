@@ -119,6 +119,7 @@ struct Tables {
   real MP[P2];
   real KP[P2];
   real WQ[Q];
+  real SQ[Q];  // square roots of WQ
   real MU[P];
   // pairs of folded entries for the packed FP32 contractions (two matrices
   // applied at once, see fwd_pm2): XE[0][i] = (FE[0][i], FE[0][i]),
@@ -153,6 +154,7 @@ __host__ __device__ constexpr bool corner_f4(int c) { return c == hpse::COEF_VER
 using hpse::MODE_PLAIN;
 using hpse::MODE_PCG;
 using hpse::MODE_TRANSPOSE;
+using hpse::MODE_RESIDUAL;
 typedef hpse::ApplyArgsT<real> ApplyArgs;
 typedef hpse::PrecArgsT<real> PrecArgs;
 
@@ -347,7 +349,7 @@ __host__ __device__ constexpr bool packed_coef(int c, int stage) {
 }
 
 // -div(a grad u) in the transpose mode (rho read from global memory) keeps
-// the scalar stages and rho in registers: the packed form measured slower there
+// the scalar stages: the packed form measured slower there
 __host__ __device__ constexpr bool packed_mode(int c, int mode) {
   return mode != hpse::MODE_TRANSPOSE || c != hpse::COEF_SCALAR;
 }
@@ -1309,7 +1311,7 @@ __global__ void __launch_bounds__(NT, APPLY_MINB) k_apply(const ApplyArgs A) {
 
   for (int t = tid; t < P2; t += nt) stab[t] = c_tab.D[t];
   FaceMeta *fm = face_meta(stab);
-  if (MODE != MODE_TRANSPOSE && tid < 6) face_meta_fill<COEF, MODE>(A, e, r, geo_e, fm, tid);
+  if ((MODE == MODE_PLAIN || MODE == MODE_PCG) && tid < 6) face_meta_fill<COEF, MODE>(A, e, r, geo_e, fm, tid);
   if (MODE != MODE_TRANSPOSE) {
     if (MODE == MODE_PCG) {
       const double bt = A.beta[A.prob[e] * A.n_rhs + r];
@@ -1432,13 +1434,33 @@ __global__ void __launch_bounds__(NT, APPLY_MINB) k_apply(const ApplyArgs A) {
     const real sz2c =
         (COEF == COEF_EDGE || COEF == COEF_VERTEX_EDGE) ? sz2 * A.kappa[(int64_t)e * hpse::KAPPA_STRIDE + qa] : sz2;
     // lanes past the last column keep their rho in the spare column Q2
-    constexpr bool inplace = L::RHO_INPLACE && packed_mode(COEF, MODE);
+    constexpr bool inplace = L::RHO_INPLACE;
     std::conditional_t<inplace, ColumnRhoT<TS>, ColumnRho<L::RHO_SMEM>> rho;
     if constexpr (inplace) rho.bind(sT, l, ok);
     else rho.bind(srho, ok ? l : Q2);
+    // -sqrt(w J) of the column's points but for its factor along z (residual map and its transpose)
+    real swab = 0;
+    if (MODE == MODE_RESIDUAL || (MODE == MODE_TRANSPOSE && A.zin)) swab = -c_tab.SQ[qa] * c_tab.SQ[qb] * A.sqj[e];
+    auto emit = [&](int q, real sigma) {  // sigma: L u = -a sigma
+      const int64_t o = cbase + (int64_t)q * Q2;
+      real v = (real)A.f[(int64_t)r * A.nquad + o];
+      v += var_coef(COEF) ? (real)A.aux[A.nquad + o] * sigma : sigma;
+      if (ok) A.zout[(int64_t)r * A.nquad + o] = swab * c_tab.SQ[q] * v;
+    };
     if (MODE == MODE_TRANSPOSE) {
+      if (A.zin) {
 #pragma unroll
-      for (int qc = 0; qc < Q; ++qc) rho[qc] = (real)A.rho[(int64_t)r * A.nquad + cbase + (int64_t)qc * Q2];
+        for (int qc = 0; qc < Q; ++qc) {
+          const int64_t o = cbase + (int64_t)qc * Q2;
+          real v = A.zin[(int64_t)r * A.nquad + o];
+          if (var_coef(COEF)) v *= (real)A.aux[A.nquad + o];
+          rho[qc] = swab * c_tab.SQ[qc] * v;
+        }
+      } else {
+#pragma unroll
+        for (int qc = 0; qc < Q; ++qc) rho[qc] = (real)A.rho[(int64_t)r * A.nquad + cbase + (int64_t)qc * Q2];
+      }
+      __syncwarp();  // lanes past the last column read its rho
     } else if constexpr (packed_coef(COEF, 4)) {
       // -div(a grad u): A = (TL, T10) -> (p0, px) = (B0 TL, B0 T10),
       // B = (T01, T00) -> (py, p2) = (B0 T01, B2 T00), p1 = B1 T00 on B.y;
@@ -1479,9 +1501,13 @@ __global__ void __launch_bounds__(NT, APPLY_MINB) k_apply(const ApplyArgs A) {
             const real sigma0 = sz2c * b.y + a.x;
             real mq, dx, dy, dz;
             load_coef4(A.coef + 4 * (cbase + (int64_t)q * Q2), mq, dx, dy, dz);
-            rho[q] = mq * (sigma0 + dz * (p1 + sg * m1) + dx * a.y + dy * b.x);
+            const real sigma = sigma0 + dz * (p1 + sg * m1) + dx * a.y + dy * b.x;
+            if (MODE == MODE_RESIDUAL) emit(q, sigma);
+            else rho[q] = mq * sigma;
           } else {
-            rho[q] = wab * c_tab.WQ[q] * (sz2c * b.y + b.x);
+            const real sigma = sz2c * b.y + b.x;
+            if (MODE == MODE_RESIDUAL) emit(q, sigma);
+            else rho[q] = wab * c_tab.WQ[q] * sigma;
           }
         }
         __syncwarp();  // scheduling fence (register pressure); reached by all 32 lanes
@@ -1528,14 +1554,18 @@ __global__ void __launch_bounds__(NT, APPLY_MINB) k_apply(const ApplyArgs A) {
           if (var_coef(COEF)) {
             real mq, dx, dy, dz;
             load_coef4(A.coef + 4 * (cbase + (int64_t)q * Q2), mq, dx, dy, dz);
-            rho[q] = mq * (sigma0 + dz * (p1 + sg * m1) + dx * (px + sg * mx) + dy * (py + sg * my));
+            const real sigma = sigma0 + dz * (p1 + sg * m1) + dx * (px + sg * mx) + dy * (py + sg * my);
+            if (MODE == MODE_RESIDUAL) emit(q, sigma);
+            else rho[q] = mq * sigma;
           } else {
-            rho[q] = wab * c_tab.WQ[q] * sigma0;
+            if (MODE == MODE_RESIDUAL) emit(q, sigma0);
+            else rho[q] = wab * c_tab.WQ[q] * sigma0;
           }
         }
         __syncwarp();  // scheduling fence (register pressure); reached by all 32 lanes
       }
     }
+    if (MODE == MODE_RESIDUAL) continue;
     if constexpr (packed_coef(COEF, 8) && packed_mode(COEF, MODE)) {
       // -div(a grad u): (rho, d_x rho) -> (rp, xp) by (B0, B0), (d_y rho,
       // sz2 rho) -> (yp, zp) by (B0, B2), d_z rho by B1 into zp (scalar);
@@ -1649,6 +1679,7 @@ __global__ void __launch_bounds__(NT, APPLY_MINB) k_apply(const ApplyArgs A) {
       }
     }
   }
+  if (MODE == MODE_RESIDUAL) return;
   __syncthreads();
 
   // ---- y-stage transpose (lines (qa, k)), outputs j in chunks ------------

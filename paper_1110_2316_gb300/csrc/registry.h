@@ -21,7 +21,8 @@ namespace hpse {
 enum { COEF_LAPLACE = 0, COEF_SCALAR = 1, COEF_EDGE = 2, COEF_VERTEX = 3, COEF_VERTEX_EDGE = 4, COEF_GENERAL = 5 };
 // KAPPA_STRIDE = 2 * HPSE_MAX_W + 1, CSCR_STRIDE = HPSE_MAX_W + 1 (checked in the host library)
 enum { KAPPA_STRIDE = 21, CSCR_STRIDE = 11, FACE_W = 10, ZEIG_STRIDE = 132 };
-enum { MODE_PLAIN = 0, MODE_PCG = 1, MODE_TRANSPOSE = 2 };
+// MODE_RESIDUAL: z = sqrt(w J) (L u - f) at the volume points, no transpose (COEF_LAPLACE, COEF_SCALAR)
+enum { MODE_PLAIN = 0, MODE_PCG = 1, MODE_TRANSPOSE = 2, MODE_RESIDUAL = 3 };
 
 template <typename T>
 struct ApplyArgsT {
@@ -43,7 +44,14 @@ struct ApplyArgsT {
   const double *beta;
   T *pnew;
   double *partial;
-  const double *rho;
+  const double *rho;        // MODE_TRANSPOSE: the weighted point values, or null with zin
+  // residual map: w J, a at the points ([2][nquad] of the mesh's FP64 data), the
+  // source f, the point values written (MODE_RESIDUAL) or transposed (MODE_TRANSPOSE)
+  const double *aux;
+  const double *f;
+  const T *sqj;             // [E] square root of the element's Jacobian
+  T *zout;
+  const T *zin;
   int32_t skip_faces;
   int32_t self_only;        // 1: neighbour traces taken as zero (diagonal blocks of A)
   // edge neighbourhood (COEF_EDGE); null / 0 for box meshes

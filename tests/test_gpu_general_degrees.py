@@ -31,7 +31,7 @@ def _problem(W):
              [-0.2 * np.cos(x * z), 0.15 * np.cos(x - y), -1.5 + 0.3 * np.sin(x + z)]]
         return A, [0.4 * np.cos(y), -0.7 * np.sin(x), 0.25 + z], 1.3 + np.sin(x * y)
 
-    one = lambda xs, ys, zs: 1.0 + 0 * wl._grid(xs, ys, zs)[0]  # noqa: E731
+    one = lambda xs, ys, zs: wl._full(1.0, xs, ys, zs)  # noqa: E731
     return wl.Problem(mesh, [one], [one], op=op)
 
 
