@@ -48,6 +48,16 @@ def _generate():
                 with open(path, "w") as f:
                     f.write(text)
             units.append(path)
+    # second FP64 launch shape of the apply kernels (threads per CTA, see csrc/registry.h)
+    for w, nt in ((2, 128), (3, 128), (4, 192), (5, 256), (6, 128), (7, 128)):
+        path = os.path.join(GEN, f"inst_f64b_w{w}.cu")
+        text = (f"#define REAL double\n#define WDEG {w}\n#define HPSE_APPLY_NT {nt}\n#define HPSE_LINES_NC 4\n"
+                f"#define HPSE_APPLY_ONLY\n#define HPSE_REGISTER_NAME hpse_register_f64b_w{w}\n#define HPSE_DOUBLE\n"
+                f'#include "inst_template.cuh"\n')
+        if not os.path.exists(path) or open(path).read() != text:
+            with open(path, "w") as f:
+                f.write(text)
+        units.append(path)
     # the one-pass element-block products, one unit per precision
     for prec, extra in (("f32", ""), ("f64", "#define BJP_F64\n")):
         path = os.path.join(GEN, f"bj_pass_{prec}.cu")

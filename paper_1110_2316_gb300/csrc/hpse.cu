@@ -43,8 +43,15 @@ HPSE_DECL(7)
 HPSE_DECL(8)
 HPSE_DECL(9)
 HPSE_DECL(10)
+extern "C" void hpse_register_f64b_w2(KernelSet *);
+extern "C" void hpse_register_f64b_w3(KernelSet *);
+extern "C" void hpse_register_f64b_w4(KernelSet *);
+extern "C" void hpse_register_f64b_w5(KernelSet *);
+extern "C" void hpse_register_f64b_w6(KernelSet *);
+extern "C" void hpse_register_f64b_w7(KernelSet *);
 
 static KernelSet g_sets[2][HPSE_MAX_W + 1];
+static KernelSet g_alt[HPSE_MAX_W + 1];  // second FP64 launch shape of the apply kernels (hpse::alt_shape)
 static bool g_sets_ready = false;
 static long long g_launches = 0;
 
@@ -63,6 +70,9 @@ static void init_registry() {
     f64[w](&g_sets[0][w]);
     f32[w](&g_sets[1][w]);
   }
+  const RegFn alt[] = {hpse_register_f64b_w2, hpse_register_f64b_w3, hpse_register_f64b_w4,
+                       hpse_register_f64b_w5, hpse_register_f64b_w6, hpse_register_f64b_w7};
+  for (int w = hpse::ALT_W0; w <= hpse::ALT_W1; ++w) alt[w - hpse::ALT_W0](&g_alt[w]);
   g_sets_ready = true;
 }
 
@@ -182,6 +192,7 @@ struct SolverWork {
 
 struct hpse_mesh {
   int device = 0;
+  int n_sm = 1;  // SMs of the device
   int n_elem = 0, n_problem = 0, n_rhs = 0, coef_kind = 0;
   std::vector<int> W, prob, nbr;
   std::vector<double> lo, hi;
@@ -1044,6 +1055,13 @@ template <typename T>
 static hpse_status launch_curved(hpse_mesh *m, int mode, const T *u, T *y, double *partial, int n_rhs,
                                  int self_only, int only_W, cudaStream_t s);
 
+// the kernels of one degree's apply launch of `items` (element, rhs) items, one of
+// `all_items` in the degree groups that run at the same time
+static const KernelSet &apply_set(const hpse_mesh *m, int pi, int W, long long items, long long all_items) {
+  return pi == 0 && m->apply_coef != hpse::COEF_GENERAL && hpse::alt_shape(W, items, all_items, m->n_sm) ? g_alt[W]
+                                                                                                          : g_sets[pi][W];
+}
+
 template <typename T>
 static hpse_status launch_apply_all(hpse_mesh *m, int mode, ApplyArgsT<T> base_args, cudaStream_t s) {
   const int pi = sizeof(T) == 8 ? 0 : 1;
@@ -1053,7 +1071,7 @@ static hpse_status launch_apply_all(hpse_mesh *m, int mode, ApplyArgsT<T> base_a
     ApplyArgsT<T> a = base_args;
     a.elems = g.elems.as<int32_t>();
     a.n_group = g.n;
-    const KernelSet &ks = g_sets[pi][g.W];
+    const KernelSet &ks = apply_set(m, pi, g.W, (long long)g.n * m->n_rhs, n_items_all(m));
     const int th = m->threads[0][pi][g.W];
     CK(ks.apply(m->apply_coef, mode, &a, g.n * m->n_rhs, th, group_stream(m, gi, s)));
     ++g_launches;
@@ -2211,6 +2229,7 @@ extern "C" hpse_status hpse_setup_mesh(const hpse_mesh_desc *d, int device, hpse
   // ---- device ---------------------------------------------------------------
   init_registry();
   CK(cudaSetDevice(device));
+  CK(cudaDeviceGetAttribute(&m->n_sm, cudaDevAttrMultiProcessorCount, device));
   std::map<int, std::vector<int>> by_w;
   for (int e = 0; e < E; ++e) by_w[m->W[e]].push_back(e);
   for (auto &kv : by_w) {
@@ -2219,6 +2238,7 @@ extern "C" hpse_status hpse_setup_mesh(const hpse_mesh_desc *d, int device, hpse
     const hm::DegreeTables &t = m->tabs[W];
     CK(g_sets[0][W].upload(t.packed.data()));
     CK(g_sets[1][W].upload(t.packed.data()));
+    if (g_alt[W].upload) CK(g_alt[W].upload(t.packed.data()));
     Group g;
     g.W = W;
     g.n = (int)kv.second.size();
@@ -2911,10 +2931,10 @@ extern "C" hpse_status hpse_setup_block_preconditioner(hpse_mesh *m) {
     ApplyArgsT<double> a = apply_args<double>(m, g, pu.as<double>(), py.as<double>());
     a.n_rhs = nc;
     a.self_only = 1;
-    const KernelSet &ks = g_sets[0][g.W];
     const int th = m->threads[0][0][g.W];
     for (int j0 = 0; j0 < n; j0 += nc) {
       const int c = std::min(nc, n - j0);
+      const KernelSet &ks = apply_set(m, 0, g.W, (long long)g.n * c, (long long)g.n * c);
       a.n_rhs = c;
       ba.n_rhs = c;
       k_bj_probe<<<g.n * c, 128, 0, s>>>(ba, j0, c, pu.as<double>());

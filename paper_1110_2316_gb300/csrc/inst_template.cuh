@@ -1,6 +1,8 @@
 // inst_template.cuh -- launchers for one (REAL, WDEG) instantiation of
 // kernels.cuh.  A generated translation unit defines REAL, WDEG,
 // HPSE_REGISTER_NAME (and HPSE_DOUBLE for REAL = double), then includes this.
+// HPSE_APPLY_ONLY with HPSE_APPLY_NT, HPSE_LINES_NC: the apply kernels alone in a
+// second launch shape.
 #include <cmath>
 #include <vector>
 
@@ -42,10 +44,12 @@ cudaError_t apply_fn(int coef, int mode, const void *args, int n_items, int thre
     if (mode == MODE_PCG) return launch_apply_t<COEF_VERTEX_EDGE, MODE_PCG>(args, n_items, threads, s);
     if (mode == MODE_TRANSPOSE)
       return launch_apply_t<COEF_VERTEX_EDGE, MODE_TRANSPOSE>(args, n_items, threads, s);
+#if !defined(HPSE_APPLY_ONLY)
   } else if (coef == hpse::COEF_GENERAL) {
     if (mode == MODE_PLAIN) return launch_apply_gen<MODE_PLAIN>(args, n_items, s);
     if (mode == MODE_PCG) return launch_apply_gen<MODE_PCG>(args, n_items, s);
     if (mode == MODE_TRANSPOSE) return launch_apply_gen<MODE_TRANSPOSE>(args, n_items, s);
+#endif
   }
   return cudaErrorInvalidValue;
 }
@@ -62,6 +66,7 @@ size_t apply_smem_fn(int coef) {
 
 int apply_max_threads_fn(int) { return NT; }
 
+#if !defined(HPSE_APPLY_ONLY)
 template <int MODE, int ITEMS>
 cudaError_t launch_precond_t(const void *args, int n_items, cudaStream_t s) {
   typedef PcLayout<ITEMS> L;
@@ -80,6 +85,7 @@ cudaError_t precond_fn(int mode, const void *args, int n_items, int threads, cud
     return few ? launch_precond_t<MODE_PCG, 1>(args, n_items, s) : launch_precond_t<MODE_PCG, PC_ITEMS>(args, n_items, s);
   return cudaErrorInvalidValue;
 }
+#endif  // HPSE_APPLY_ONLY
 
 template <int COEF, int MODE>
 cudaError_t set_smem_attr() {
@@ -164,6 +170,7 @@ cudaError_t upload_fn(const double *pk) {
   for (int i = 0; i < P; ++i) t.MU[i] = (real)pk[o++];
   cudaError_t err = cudaMemcpyToSymbol(c_tab, &t, sizeof(Tables));
   if (err != cudaSuccess) return err;
+#if !defined(HPSE_APPLY_ONLY)
   // D_Q and D_Q^2 of the Q-point grid (integration-by-parts transpose), formed in FP64
   {
     IbpTables it;
@@ -179,6 +186,7 @@ cudaError_t upload_fn(const double *pk) {
     err = cudaMemcpyToSymbol(c_ibp, &it, sizeof(IbpTables));
     if (err != cudaSuccess) return err;
   }
+#endif  // HPSE_APPLY_ONLY
   cudaError_t e2;
   if ((e2 = set_smem_attr<COEF_LAPLACE, MODE_PLAIN>()) != cudaSuccess) return e2;
   if ((e2 = set_smem_attr<COEF_LAPLACE, MODE_PCG>()) != cudaSuccess) return e2;
@@ -197,6 +205,7 @@ cudaError_t upload_fn(const double *pk) {
   if ((e2 = set_smem_attr<COEF_VERTEX_EDGE, MODE_PLAIN>()) != cudaSuccess) return e2;
   if ((e2 = set_smem_attr<COEF_VERTEX_EDGE, MODE_PCG>()) != cudaSuccess) return e2;
   if ((e2 = set_smem_attr<COEF_VERTEX_EDGE, MODE_TRANSPOSE>()) != cudaSuccess) return e2;
+#if !defined(HPSE_APPLY_ONLY)
   if ((e2 = set_smem_attr_gen<MODE_PLAIN>()) != cudaSuccess) return e2;
   if ((e2 = set_smem_attr_gen<MODE_PCG>()) != cudaSuccess) return e2;
   if ((e2 = set_smem_attr_gen<MODE_TRANSPOSE>()) != cudaSuccess) return e2;
@@ -208,9 +217,11 @@ cudaError_t upload_fn(const double *pk) {
   if ((e2 = cudaFuncSetAttribute(k_precond<MODE_PCG, PC_ITEMS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)PcLayout<PC_ITEMS>::BYTES)) != cudaSuccess)
     return e2;
+#endif  // HPSE_APPLY_ONLY
   return cudaSuccess;
 }
 
+#if !defined(HPSE_APPLY_ONLY)
 cudaError_t transpose_ibp_fn(int coef, const void *args, int n_items, cudaStream_t s) {
   if (n_items <= 0) return cudaSuccess;
   if (coef == COEF_LAPLACE) return launch_transpose_ibp_t<COEF_LAPLACE>(args, n_items, s);
@@ -223,6 +234,8 @@ size_t ibp_smem_fn(int coef) {
   if (coef == COEF_SCALAR) return IbpLayout<COEF_SCALAR>::FITS ? IbpLayout<COEF_SCALAR>::BYTES : 0;
   return 0;
 }
+
+#endif  // HPSE_APPLY_ONLY
 
 static_assert(ApplyLayout<COEF_SCALAR>::BYTES <= 232448, "apply kernel exceeds 227 KB of shared memory");
 
@@ -239,7 +252,9 @@ extern "C" void HPSE_REGISTER_NAME(hpse::KernelSet *ks) {
   ks->apply = apply_fn;
   ks->apply_smem = apply_smem_fn;
   ks->apply_max_threads = apply_max_threads_fn;
+#if !defined(HPSE_APPLY_ONLY)
   ks->precond = precond_fn;
   ks->transpose_ibp = transpose_ibp_fn;
   ks->ibp_smem = ibp_smem_fn;
+#endif
 }

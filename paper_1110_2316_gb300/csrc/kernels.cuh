@@ -74,15 +74,18 @@ __host__ __device__ constexpr bool odd_pp(int t) { return t < 2; }
 // whole warps, capped; every stage then runs at most once per thread when
 // Q^2 <= NT, so no constant-table read is loop-invariant across line
 // iterations and every FMA keeps its constant-bank operand.
+// (FP64: 256, two passes over the z-lines from W = 8 on, where a CTA is alone on
+// its SM and 255 registers pay; at W = 8 one pass of 320 threads is faster, 864
+// -> 819 us for 1,024 items, at W = 9 and 10 it is slower by 2 to 6 %.)
 #if defined(HPSE_DOUBLE)
-#define HPSE_APPLY_MAXT 256
+#define HPSE_APPLY_MAXT (WDEG == 8 ? 320 : 256)
 #else
 #define HPSE_APPLY_MAXT 448
 #endif
 #define PAD32(n) ((((n) + 31) / 32) * 32)
 constexpr int NT_RAW = PAD32(Q2);
 #if defined(HPSE_APPLY_NT)
-constexpr int NT = HPSE_APPLY_NT;  // set at build time (launch-shape experiments)
+constexpr int NT = HPSE_APPLY_NT;  // set by the unit (second FP64 launch shape, see registry.h)
 #else
 constexpr int NT = NT_RAW < 64 ? 64 : (NT_RAW > HPSE_APPLY_MAXT ? HPSE_APPLY_MAXT : NT_RAW);
 #endif
@@ -230,7 +233,7 @@ struct Lines {
   static constexpr int PADL = PAD32(L);
   static constexpr int NC_RAW = NT / PADL;
 #if defined(HPSE_LINES_NC)
-  static constexpr int NC_MAX = HPSE_LINES_NC;  // set at build time (launch-shape experiments)
+  static constexpr int NC_MAX = HPSE_LINES_NC;  // set by the unit, with HPSE_APPLY_NT
 #else
   static constexpr int NC_MAX = 2;
 #endif

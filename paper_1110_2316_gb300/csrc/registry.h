@@ -96,6 +96,23 @@ inline int packed_table_size(int W) {
   return 3 * Q * P + 4 * P * P + Q + P + Q * Q;
 }
 
+// Second FP64 launch shape of the apply kernels (units f64b, HPSE_APPLY_ONLY):
+// the threads per CTA that suit the other end of the item counts than the
+// first one.  W = 2..5: more threads (128, 128, 192, 256 for 64, 64, 96, 128),
+// for launches of at most one item per SM, where an item's latency counts and
+// the extra warps shorten the line stages and the face phase (Laplacian / variable
+// coefficient, one item per SM: W = 3 22.7 -> 18.7 / 31.0 -> 26.8 us, W = 4 31.5 ->
+// 24.8 / 45.4 -> 37.1); with two and more items per SM they cost up to 20 %.
+// W = 6, 7: fewer (128 for 192, 256), for launches of more items than SMs, where
+// the registers then allow two CTAs per SM and one's barriers hide behind the
+// other (1,024 items: W = 6 387 -> 346 / 605 -> 564 us, W = 7 537 -> 503 / 887 ->
+// 843); a lone item is slower (57.6 -> 65.7 us).
+constexpr int ALT_W0 = 2, ALT_W1 = 7;
+inline bool alt_shape(int W, long long items, long long all_items, int sms) {
+  if (W < ALT_W0 || W > ALT_W1) return false;
+  return W <= 5 ? all_items <= sms : items > sms;  // all_items: over every degree of the launch
+}
+
 struct KernelSet {
   int W;
   int is_double;
