@@ -376,38 +376,50 @@ __global__ void __launch_bounds__(TR *TC) k_bj_tri(BjArgs A, const T *X, const T
   }
 }
 
+// Vector kernels of the PCG step, one warp per (element, rhs) item, eight items
+// per CTA: the FP64 sums are bound by the FP64 pipe, and a warp that keeps its
+// item's whole sum adds five values in the end, where a CTA per item added five
+// per warp (config 2, 16 rhs: 46 + 48 us for the pair, HBM 21 + 7).
+constexpr int BJ_VEC_ITEMS = 8;
+inline unsigned bj_vec_grid(int items) { return (unsigned)((items + BJ_VEC_ITEMS - 1) / BJ_VEC_ITEMS); }
+
 // PCG update x += alpha p, r -= alpha q on the group's blocks, partial r.r per
-// (element, rhs).  grid: n_group * n_rhs.
+// (element, rhs).  grid: bj_vec_grid(n_group * n_rhs), 32 * BJ_VEC_ITEMS threads.
 template <typename T>
-__global__ void k_bj_update(BjArgs A, const int32_t *prob, const double *alpha, T *x, T *r, const T *p, const T *q,
-                            double *part_rr) {
-  const int item = blockIdx.x;
+__global__ void __launch_bounds__(32 * BJ_VEC_ITEMS)
+    k_bj_update(BjArgs A, const int32_t *prob, const double *alpha, T *x, T *r, const T *p, const T *q, double *part_rr) {
+  const int item = blockIdx.x * BJ_VEC_ITEMS + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (item >= A.n_group * A.n_rhs) return;
   const int ge = item / A.n_rhs, rr = item - ge * A.n_rhs;
   const int e = A.elems[ge];
   const int64_t base = (int64_t)rr * A.ndof + A.dof_off[e];
   const T al = (T)alpha[prob[e] * A.n_rhs + rr];
   double s = 0.0;
-  for (int t = threadIdx.x; t < A.n; t += blockDim.x) {
+#pragma unroll 4
+  for (int t = lane; t < A.n; t += 32) {
     if (x) x[base + t] += al * p[base + t];
     const T v = r[base + t] - al * q[base + t];
     r[base + t] = v;
-    s += (double)v * (double)v;
+    const double w = hpse::widen(v);
+    s += w * w;
   }
-  s = block_sum_d(s);
-  if (threadIdx.x == 0) part_rr[(int64_t)e * A.n_rhs + rr] = s;
+  s = warp_sum(s);
+  if (lane == 0) part_rr[(int64_t)e * A.n_rhs + rr] = s;
 }
 
-// partial z.r per (element, rhs) on the group's blocks.  grid: n_group * n_rhs.
+// partial z.r per (element, rhs) on the group's blocks.  grid and threads as k_bj_update.
 template <typename T>
-__global__ void k_bj_dot(BjArgs A, const T *z, const T *r, double *part) {
-  const int item = blockIdx.x;
+__global__ void __launch_bounds__(32 * BJ_VEC_ITEMS) k_bj_dot(BjArgs A, const T *z, const T *r, double *part) {
+  const int item = blockIdx.x * BJ_VEC_ITEMS + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (item >= A.n_group * A.n_rhs) return;
   const int ge = item / A.n_rhs, rr = item - ge * A.n_rhs;
   const int e = A.elems[ge];
   const int64_t base = (int64_t)rr * A.ndof + A.dof_off[e];
   double s = 0.0;
-  for (int t = threadIdx.x; t < A.n; t += blockDim.x) s += (double)z[base + t] * (double)r[base + t];
-  s = block_sum_d(s);
-  if (threadIdx.x == 0) part[(int64_t)e * A.n_rhs + rr] = s;
+#pragma unroll 4
+  for (int t = lane; t < A.n; t += 32) s += hpse::widen(z[base + t]) * hpse::widen(r[base + t]);
+  s = warp_sum(s);
+  if (lane == 0) part[(int64_t)e * A.n_rhs + rr] = s;
 }
 
 // Shapes of the two triangular products, picked per degree group and precision

@@ -55,7 +55,7 @@ constexpr int GEN_MINB = sizeof(real) == 8 ? 1 : (640 / NT < 1 ? 1 : (640 / NT >
 struct GenLayout {
   static constexpr int TS = t_stride(3, 6, GEN_MINB);  // row stride of the T fields
   static constexpr int TF = TS * P;
-  static constexpr size_t RED_OFF = apply_bytes(3, 6, TS) - 64 * sizeof(double);
+  static constexpr size_t RED_OFF = red_in_x(3) ? X_OFF : apply_bytes(3, 6, TS) - NT * sizeof(double);
   static constexpr int T_NEED = P3 + 6 * FACE_ARR * P2;
   static constexpr int T_REGION = 6 * TF > T_NEED ? 6 * TF : T_NEED;
   static constexpr size_t BYTES = apply_bytes(3, 6, TS);
@@ -472,7 +472,7 @@ __global__ void __launch_bounds__(NT, GEN_MINB) k_apply_gen(const ApplyArgs A) {
   for (int t = tid; t < P3; t += nt) {
     const real v = sy[t];
     A.y[base + t] = v;
-    if (MODE == MODE_PCG) part += (double)v * (double)su[t];
+    if (MODE == MODE_PCG) part += hpse::widen(v) * hpse::widen(su[t]);
   }
   if (MODE == MODE_PCG) {
     const double s = block_sum(part, red);

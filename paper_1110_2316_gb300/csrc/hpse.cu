@@ -220,6 +220,7 @@ struct hpse_mesh {
   std::vector<int64_t> bface_off;          // offset of each face's Q^2 points
   int64_t nface_pts = 0;
   std::vector<int> prob_ptr, prob_elems;   // CSR of elements per problem
+  int max_prob_items = 0;                  // the longest row
   std::map<int, hm::DegreeTables> tabs;
   std::vector<Group> groups;
   // device mesh arrays
@@ -346,7 +347,7 @@ __global__ void k_dot(ElemVecArgs A, const TA *a, const TB *b, double *part) {
   const int n = A.item_n[e];
   const int64_t base = (int64_t)r * A.ndof + A.dof_off[e];
   double s = 0.0;
-  for (int t = threadIdx.x; t < n; t += blockDim.x) s += (double)a[base + t] * (double)b[base + t];
+  for (int t = threadIdx.x; t < n; t += blockDim.x) s += hpse::widen(a[base + t]) * hpse::widen(b[base + t]);
   s = block_sum_d(s);
   if (threadIdx.x == 0) part[(int64_t)e * A.n_rhs + r] = s;
 }
@@ -461,12 +462,26 @@ __device__ double fin_sum(const FinArgs &F, const double *part, int p, int r) {
   return block_sum_d(s);
 }
 
+// The two scalar kernels of every PCG iteration sum a problem's partials with one
+// warp per (problem, rhs), four per CTA, where no problem has more than
+// FIN_WARP_ITEMS items (WARP; a batch of small problems: 4.1 + 7.1 us a pair for
+// 1,024 problems of 8 elements with a CTA per problem and sum), else with a CTA each.
+constexpr int FIN_WARP_ITEMS = 64;
+constexpr int FIN_PER_CTA = 4;
+__device__ __forceinline__ double fin_warp_sum(const FinArgs &F, const double *part, int b, int e_, int r) {
+  double s = 0.0;
+  for (int i = b + (threadIdx.x & 31); i < e_; i += 32) s += part[(int64_t)F.prob_elems[i] * F.n_rhs + r];
+  return warp_sum(s);
+}
+
 // after q = A p: alpha = rz / (p.q)
-__global__ void k_fin_alpha(FinArgs F, Scalars S, const double *part_pq) {
-  const int pr = blockIdx.x;
+template <bool WARP>
+__global__ void __launch_bounds__(128) k_fin_alpha(FinArgs F, Scalars S, const double *part_pq, int npr) {
+  const int pr = WARP ? blockIdx.x * FIN_PER_CTA + (threadIdx.x >> 5) : blockIdx.x;
+  if (pr >= npr) return;
   const int p = pr / F.n_rhs, r = pr - p * F.n_rhs;
-  const double pq = fin_sum(F, part_pq, p, r);
-  if (threadIdx.x == 0) {
+  const double pq = WARP ? fin_warp_sum(F, part_pq, F.prob_ptr[p], F.prob_ptr[p + 1], r) : fin_sum(F, part_pq, p, r);
+  if ((WARP ? threadIdx.x & 31 : threadIdx.x) == 0) {
     S.pq[pr] = pq;
     double a = 0.0;
     if (S.active[pr]) {
@@ -487,12 +502,37 @@ __global__ void k_fin_alpha(FinArgs F, Scalars S, const double *part_pq) {
 }
 
 // after the update + preconditioner: convergence test and beta
-__global__ void k_fin_beta(FinArgs F, Scalars S, const double *part_rr, const double *part_rz) {
-  const int pr = blockIdx.x;
+template <bool WARP>
+__global__ void __launch_bounds__(128)
+    k_fin_beta(FinArgs F, Scalars S, const double *part_rr, const double *part_rz, int npr) {
+  const int pr = WARP ? blockIdx.x * FIN_PER_CTA + (threadIdx.x >> 5) : blockIdx.x;
+  if (pr >= npr) return;
   const int p = pr / F.n_rhs, r = pr - p * F.n_rhs;
-  const double rr = fin_sum(F, part_rr, p, r);
-  const double rz = fin_sum(F, part_rz, p, r);
-  if (threadIdx.x == 0) {
+  double rr, rz;
+  if (WARP) {
+    const int b = F.prob_ptr[p], e_ = F.prob_ptr[p + 1];
+    rr = fin_warp_sum(F, part_rr, b, e_, r);
+    rz = fin_warp_sum(F, part_rz, b, e_, r);
+  } else {
+    // both sums in one sweep and one reduction
+    __shared__ double red[2][4];
+    double a = 0.0, c = 0.0;
+    for (int i = F.prob_ptr[p] + threadIdx.x; i < F.prob_ptr[p + 1]; i += blockDim.x) {
+      const int64_t o = (int64_t)F.prob_elems[i] * F.n_rhs + r;
+      a += part_rr[o];
+      c += part_rz[o];
+    }
+    a = warp_sum(a);
+    c = warp_sum(c);
+    if ((threadIdx.x & 31) == 0) {
+      red[0][threadIdx.x >> 5] = a;
+      red[1][threadIdx.x >> 5] = c;
+    }
+    __syncthreads();
+    rr = red[0][0] + red[0][1] + red[0][2] + red[0][3];
+    rz = red[1][0] + red[1][1] + red[1][2] + red[1][3];
+  }
+  if ((WARP ? threadIdx.x & 31 : threadIdx.x) == 0) {
     double b = 0.0;
     if (S.active[pr]) {
       S.iters[pr] += 1;
@@ -1237,7 +1277,7 @@ static hpse_status launch_bj_all(hpse_mesh *m, int mode, const PrecArgsT<T> &b, 
     const int items = g.n * b.n_rhs;
     const T *rin = mode == MODE_PCG ? b.r : b.rin;
     if (mode == MODE_PCG) {
-      k_bj_update<T><<<items, 128, 0, gs>>>(a, b.prob, b.alpha, b.x, b.r, b.p, b.q, b.part_rr);
+      k_bj_update<T><<<bj_vec_grid(items), 32 * BJ_VEC_ITEMS, 0, gs>>>(a, b.prob, b.alpha, b.x, b.r, b.p, b.q, b.part_rr);
       CK(cudaGetLastError());
       g_launches += 2;
     }
@@ -1257,7 +1297,7 @@ static hpse_status launch_bj_all(hpse_mesh *m, int mode, const PrecArgsT<T> &b, 
       g_launches += 2;
     }
     if (mode == MODE_PCG) {
-      k_bj_dot<T><<<items, 128, 0, gs>>>(a, b.zout, b.r, b.part_rz);
+      k_bj_dot<T><<<bj_vec_grid(items), 32 * BJ_VEC_ITEMS, 0, gs>>>(a, b.zout, b.r, b.part_rz);
       CK(cudaGetLastError());
     }
   }
@@ -2215,7 +2255,10 @@ extern "C" hpse_status hpse_setup_mesh(const hpse_mesh_desc *d, int device, hpse
   m->prob_ptr.assign(m->n_problem + 1, 0);
   for (int e = 0; e < E; ++e) m->prob_ptr[m->prob[e] + 1]++;
   for (int c = 0; c < C; ++c) m->prob_ptr[m->cprob[c] + 1]++;
-  for (int p = 0; p < m->n_problem; ++p) m->prob_ptr[p + 1] += m->prob_ptr[p];
+  for (int p = 0; p < m->n_problem; ++p) {
+    m->max_prob_items = std::max(m->max_prob_items, m->prob_ptr[p + 1]);
+    m->prob_ptr[p + 1] += m->prob_ptr[p];
+  }
   {
     std::vector<int> fill(m->prob_ptr.begin(), m->prob_ptr.end() - 1);
     m->prob_elems.assign(E + C, 0);
@@ -3233,7 +3276,10 @@ static hpse_status pcg_iteration(hpse_mesh *m, T *x, T *r, T *z, T *pin, T *pout
   a.partial = w.part0.as<double>();
   hpse_status st = launch_apply_all<T>(m, MODE_PCG, a, s);
   if (st != HPSE_OK) return st;
-  k_fin_alpha<<<npr, 128, 0, s>>>(fin_args(m), S, w.part0.as<double>());
+  const bool fw = m->max_prob_items <= FIN_WARP_ITEMS;
+  const int fg = fw ? (npr + FIN_PER_CTA - 1) / FIN_PER_CTA : npr;
+  if (fw) k_fin_alpha<true><<<fg, 128, 0, s>>>(fin_args(m), S, w.part0.as<double>(), npr);
+  else k_fin_alpha<false><<<fg, 128, 0, s>>>(fin_args(m), S, w.part0.as<double>(), npr);
   CK(cudaGetLastError());
   ++g_launches;
   PrecArgsT<T> pa = prec_args<T>(m, m->groups[0]);
@@ -3247,7 +3293,8 @@ static hpse_status pcg_iteration(hpse_mesh *m, T *x, T *r, T *z, T *pin, T *pout
   pa.part_rz = w.part2.as<double>();
   st = launch_prec_all<T>(m, MODE_PCG, pa, s);
   if (st != HPSE_OK) return st;
-  k_fin_beta<<<npr, 128, 0, s>>>(fin_args(m), S, w.part1.as<double>(), w.part2.as<double>());
+  if (fw) k_fin_beta<true><<<fg, 128, 0, s>>>(fin_args(m), S, w.part1.as<double>(), w.part2.as<double>(), npr);
+  else k_fin_beta<false><<<fg, 128, 0, s>>>(fin_args(m), S, w.part1.as<double>(), w.part2.as<double>(), npr);
   CK(cudaGetLastError());
   ++g_launches;
   return HPSE_OK;

@@ -169,20 +169,21 @@ __device__ __forceinline__ int fidx(int a, int n, int p1, int p2) {
   return (n * P + p2) * P + p1;               // (i=p1, j=p2, k=n)
 }
 
-template <typename T>
-__device__ __forceinline__ double block_sum(T v, double *red) {
-  double s = (double)v;
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int nw = (blockDim.x + 31) >> 5;
+// sum over the CTA (valid in thread 0); buf: NT doubles of shared memory that no
+// thread uses any more.  One warp adds the NT values: NT / 32 + 5 FP64 additions
+// per lane of it, where a shuffle tree in every warp takes five per warp of the CTA.
+__device__ __forceinline__ double block_sum(double v, double *buf) {
+  const int tid = threadIdx.x;
+  buf[tid] = v;
   __syncthreads();
-  if (lane == 0) red[wid] = s;
-  __syncthreads();
-  double t = 0.0;
-  if (threadIdx.x == 0) {
-    for (int i = 0; i < nw; ++i) t += red[i];
+  double s = 0.0;
+  if (tid < 32) {
+#pragma unroll
+    for (int i = 0; i < NT / 32; ++i) s += buf[tid + 32 * i];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   }
-  return t;  // valid in thread 0
+  return s;
 }
 
 // vector load of the 4 pointwise coefficients (m, d_x, d_y, d_z) of a point
@@ -845,11 +846,15 @@ __device__ __forceinline__ FaceMeta *face_meta(real *stab) {
 // warp's addresses distinct, where the padding costs no resident CTA
 // (config 2's apply 418 -> 410 us at 16 rhs, W = 7 306 -> 288 us).
 constexpr int T_PAD = sizeof(real) == 4 ? (((Q - Q2) % 32) + 32) % 32 : 0;
+// the FP64 reduction of PCG's p.q uses the X fields, free by then, where they
+// hold NT doubles, else NT doubles after everything else
+constexpr size_t X_OFF = ((size_t)P3 * sizeof(real) + 7) / 8 * 8;
+constexpr bool red_in_x(int nx) { return (size_t)(P3 + nx * QP2) * sizeof(real) >= X_OFF + NT * sizeof(double); }
 // dynamic shared memory of an apply CTA: su | NX X fields | T region | D, face data | reduction
 constexpr size_t apply_bytes(int nx, int ntf, int ts) {
   const int t = ntf * ts * P, need = P3 + 6 * FACE_ARR * P2;
   const size_t tot = (size_t)(P3 + nx * QP2 + (t > need ? t : need) + P2 + FACE_META_REALS);
-  return ((tot * sizeof(real) + 15) / 16) * 16 + 64 * sizeof(double);
+  return ((tot * sizeof(real) + 15) / 16) * 16 + (red_in_x(nx) ? 0 : NT * sizeof(double));
 }
 constexpr int sm_ctas(size_t bytes, int most) {
   const int n = (int)(233472 / (bytes + 1024));
@@ -1303,8 +1308,9 @@ struct ApplyLayout {
 #endif
   static constexpr int TOTAL = TOTAL0 + (RHO_SMEM ? RHO_LEN : 0);
   // the FP64 reduction buffer starts on a 16-byte boundary whatever REAL is
-  static constexpr size_t RED_OFF = (((size_t)TOTAL * sizeof(real) + 15) / 16) * 16;
-  static constexpr size_t BYTES = RED_OFF + 64 * sizeof(double);
+  static constexpr size_t END = (((size_t)TOTAL * sizeof(real) + 15) / 16) * 16;
+  static constexpr size_t RED_OFF = red_in_x(NX) ? X_OFF : END;
+  static constexpr size_t BYTES = END + (red_in_x(NX) ? 0 : NT * sizeof(double));
 };
 
 template <int COEF, int MODE>
@@ -1317,7 +1323,7 @@ __global__ void __launch_bounds__(NT, APPLY_MINB) k_apply(const ApplyArgs A) {
   real *stab = sT + L::T_REGION;    // D (runtime-indexed copy for the face gather) | per-face scales
   real *srho = stab + L::TABS;      // rho of the z-stage (L::RHO_SMEM)
   double *red = reinterpret_cast<double *>(smem_raw + L::RED_OFF);
-  static_assert(L::RED_OFF % 16 == 0, "reduction buffer must be 16-byte aligned");
+  static_assert(L::RED_OFF % 8 == 0, "reduction buffer must be 8-byte aligned");
   real *X0 = sX, *X2 = sX + QP2, *X1 = sX + 2 * QP2;
   constexpr int TS = L::TS, TF = TS * P;
   real *T00 = sT, *TL = sT + TF, *T10 = sT + 2 * TF, *T01 = sT + 3 * TF;
@@ -1762,7 +1768,7 @@ __global__ void __launch_bounds__(NT, APPLY_MINB) k_apply(const ApplyArgs A) {
   for (int t = tid; t < P3; t += nt) {
     const real v = sy[t];
     A.y[base + t] = v;
-    if (MODE == MODE_PCG) part += (double)v * (double)su[t];
+    if (MODE == MODE_PCG) part += hpse::widen(v) * hpse::widen(su[t]);
   }
   if (MODE == MODE_PCG) {
     const double s = block_sum(part, red);

@@ -7,6 +7,27 @@
 
 namespace hpse {
 
+// FP32 -> FP64, exact, by moving the bits: the conversion instruction runs on the
+// FP64 pipe (two lanes per clock and SM) and would bound the FP64 sums of FP32
+// vectors.  Subnormals go through an exact FP32 scaling by 2^24.
+__device__ __forceinline__ double widen(float v) {
+  const uint32_t b = __float_as_uint(v), s = b & 0x80000000u, a = b & 0x7fffffffu;
+  uint32_t hi = (a >> 3) + 0x38000000u, lo = b << 29;  // exponent bias 127 -> 1023
+  if (a - 0x00800000u >= 0x7f000000u) {                // zero, subnormal, infinity, NaN
+    if (a >= 0x7f800000u) {
+      hi = (a >> 3) + 0x70000000u;
+    } else if (a == 0) {
+      hi = lo = 0;
+    } else {
+      const uint32_t u = __float_as_uint(__uint_as_float(a) * 16777216.f);
+      hi = (u >> 3) + 0x38000000u - (24u << 20);
+      lo = u << 29;
+    }
+  }
+  return __hiloint2double((int)(s | hi), (int)lo);
+}
+__device__ __forceinline__ double widen(double v) { return v; }
+
 // COEF_EDGE: -(u_11 + u_22 + kappa(x_1) u_33) in the edge neighbourhood's
 // modified coordinates, kappa = e^{2 tau} per x-point of the element
 // COEF_VERTEX: the variable-coefficient form with per-point weights and
