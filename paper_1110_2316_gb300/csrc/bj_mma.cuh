@@ -4,7 +4,7 @@
 // FMAs and their shared loads bound the pass (271 and 480 us for 512 blocks of
 // 729); the matrix instructions cut the issued instructions, so that what is
 // left is the reading of X, its split and the latency of a block (242 and
-// 365 us; the two-product tiles took 470 and 871 us).  mma.sync and not
+// 359 us; the two-product tiles took 470 and 871 us).  mma.sync and not
 // tcgen05: the operand is a triangular, unaligned packed row block that is read
 // once, at N = 8 or 16.
 //
@@ -18,20 +18,21 @@
 // padding: consecutive triangular numbers are distinct modulo 2^k, so lanes on
 // 8 rows x columns 8 apart (t), or 4 rows x columns 4 apart (z), touch 32
 // different banks.  r is kept as ready B fragments (hi, hi, lo, lo of the two
-// k's of a lane), t of the block likewise; z stays in the accumulator layout.
+// k's of a lane), or as FP32 values split at each use where those do not fit; t
+// of the block likewise; z stays in the accumulator layout.
 // Block b + 1's t is formed in the same barrier interval as block b's z.
 #pragma once
 #include "bj_pass.cuh"
 
 // shared memory: X stages | r fragments | partial t | t fragments
-template <int NT8, int NW>
+template <int NT8, int NW, bool PRE>
 struct BjmLayout {
   static constexpr int RT = 8 * NT8;
   __host__ __device__ static int chunks(int n) { return (n + 31) / 32; }
   // floats of one X stage: 16 rows of up to n16 entries and the 16-byte slack at both ends
   __host__ __device__ static int stage(int n) { return BJP_BR * (((n + BJP_BR - 1) / BJP_BR) * BJP_BR) + 8; }
   __host__ __device__ static size_t bytes(int n, int stages) {
-    return sizeof(float) * ((size_t)stages * stage(n) + (size_t)chunks(n) * 4 * NT8 * 128 + (size_t)NW * BJP_BR * RT +
+    return sizeof(float) * ((size_t)stages * stage(n) + (size_t)chunks(n) * 4 * NT8 * (PRE ? 128 : 64) + (size_t)NW * BJP_BR * RT +
                             2 * NT8 * 128);
   }
 };
@@ -56,12 +57,24 @@ __device__ __forceinline__ float bjm_lds(uint32_t addr) {
   asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
   return v;
 }
-__device__ __forceinline__ float4 bjm_lds4(uint32_t addr) {
+// B fragment i of r (hi, hi, lo, lo of the two k's of a lane): kept split (PRE), or as
+// the FP32 values and split here
+template <bool PRE>
+__device__ __forceinline__ float4 bjm_frag(uint32_t rf, int i, int lane) {
   float4 v;
-  asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
-               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
-               : "r"(addr)
-               : "memory");
+  if constexpr (PRE) {
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                 : "r"(rf + 16 * (32 * i + lane))
+                 : "memory");
+  } else {
+    float x, y;
+    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(x), "=f"(y) : "r"(rf + 8 * (32 * i + lane)) : "memory");
+    uint32_t h0, l0, h1, l1;
+    bjm_split(x, h0, l0);
+    bjm_split(y, h1, l1);
+    v = make_float4(__uint_as_float(h0), __uint_as_float(h1), __uint_as_float(l0), __uint_as_float(l1));
+  }
   return v;
 }
 // the six products of two k-steps of one n8 tile (A hi/lo, B = (hi, hi, lo, lo) of the step), small terms apart
@@ -85,7 +98,7 @@ __device__ __forceinline__ void bjm_prod(const uint32_t (&ah)[2][4], const uint3
 
 // t = X r on one unit u of 16 columns of the block's 16 rows, added to acc.
 // x0, x1: shared addresses of (row g or g + 8, column 8 t); lane column 32 (u / 2) + 4 (u % 2) + 8 t + 2 s2 + h
-template <int NT8, bool GUARD>
+template <int NT8, bool PRE, bool GUARD>
 __device__ __forceinline__ void bjm_fwd(uint32_t x0, uint32_t x1, uint32_t rf, int i0, int dn, int u, int lane,
                                         float (&acc)[NT8][4]) {
   const int k0 = 32 * (u >> 1) + 4 * (u & 1);
@@ -106,8 +119,7 @@ __device__ __forceinline__ void bjm_fwd(uint32_t x0, uint32_t x1, uint32_t rf, i
     }
 #pragma unroll
   for (int q = 0; q < NT8; ++q)
-    bjm_prod(ah, al, bjm_lds4(rf + 16 * ((2 * u * NT8 + q) * 32 + lane)),
-             bjm_lds4(rf + 16 * (((2 * u + 1) * NT8 + q) * 32 + lane)), acc[q]);
+    bjm_prod(ah, al, bjm_frag<PRE>(rf, 2 * u * NT8 + q, lane), bjm_frag<PRE>(rf, (2 * u + 1) * NT8 + q, lane), acc[q]);
 }
 
 // z += X^T t on one group of 32 columns; ro: shared addresses of (row 8 s2 + 4 h + t, column 4 g)
@@ -136,18 +148,18 @@ __device__ __forceinline__ void bjm_back(const uint32_t (&ro)[2][2], const float
   }
 }
 
-template <int NT8, int NW, int CG>
+template <int NT8, int NW, int CG, bool PRE>
 __global__ void __launch_bounds__(32 * NW, NW >= 16 ? 1 : 16 / NW)
     k_bj_mma(BjArgs A, const float *X, const float *in, float *out, int stages, int cs, int32_t *err) {
-  typedef BjmLayout<NT8, NW> L;
+  typedef BjmLayout<NT8, NW, PRE> L;
   constexpr int RT = L::RT, NTH = 32 * NW;
   extern __shared__ __align__(16) unsigned char bjm_raw[];
   __shared__ __align__(8) uint64_t bar[2];
   __shared__ int s_bad;
   const int n = A.n, nch = L::chunks(n), stage = L::stage(n);
   float *Xs = reinterpret_cast<float *>(bjm_raw);
-  float4 *rf = reinterpret_cast<float4 *>(Xs + (size_t)stages * stage);  // [chunk][k-step][n8][lane]
-  float *ps = reinterpret_cast<float *>(rf + (size_t)nch * 4 * NT8 * 32);  // [warp][16][RT]
+  float *rf = Xs + (size_t)stages * stage;                // [chunk][k-step][n8][lane] of 4 (PRE) or 2 floats
+  float *ps = rf + (size_t)nch * NT8 * (PRE ? 512 : 256);  // [warp][16][RT]
   float4 *ts = reinterpret_cast<float4 *>(ps + NW * BJP_BR * RT);          // [k-step][n8][lane]
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int rank = blockIdx.x % cs, ge = blockIdx.x / cs;
@@ -186,11 +198,16 @@ __global__ void __launch_bounds__(32 * NW, NW >= 16 ? 1 : 16 / NW)
     const float *src = in + (int64_t)(r0 + q) * A.ndof + vb;
     const bool ok = r0 + q < A.n_rhs;
     const float v0 = ok && k < n ? src[k] : 0.f, v1 = ok && k + 1 < n ? src[k + 1] : 0.f;
-    uint32_t h0, l0, h1, l1;
-    bjm_split(v0, h0, l0);
-    bjm_split(v1, h1, l1);
-    rf[((size_t)(4 * c + s) * NT8 + (q >> 3)) * 32 + (q & 7) * 4 + t] =
-        make_float4(__uint_as_float(h0), __uint_as_float(h1), __uint_as_float(l0), __uint_as_float(l1));
+    const size_t at = ((size_t)(4 * c + s) * NT8 + (q >> 3)) * 32 + (q & 7) * 4 + t;
+    if constexpr (PRE) {
+      uint32_t h0, l0, h1, l1;
+      bjm_split(v0, h0, l0);
+      bjm_split(v1, h1, l1);
+      reinterpret_cast<float4 *>(rf)[at] =
+          make_float4(__uint_as_float(h0), __uint_as_float(h1), __uint_as_float(l0), __uint_as_float(l1));
+    } else {
+      reinterpret_cast<float2 *>(rf)[at] = make_float2(v0, v1);
+    }
   }
   __syncthreads();
 
@@ -268,10 +285,12 @@ __global__ void __launch_bounds__(32 * NW, NW >= 16 ? 1 : 16 / NW)
       for (int i = 0; i < 4; ++i) acc[q][i] = 0.f;
     const int nu = 2 * ((i0 + dn + 31) / 32);
     const int nfull = dn == BJP_BR ? 2 * ((i0 + 1) / 32) : 0;  // units wholly left of the diagonal
-    int u = warp;
+    // in reverse warp order at 16 right-hand sides: the first warps have the most columns
+    // of the other product (365 -> 359 us, 512 blocks of 729; at 8 no gain)
+    int u = NT8 == 2 ? NW - 1 - warp : warp;
 #pragma unroll 2
-    for (; u < nfull; u += NW) bjm_fwd<NT8, false>(x0, x1, rfa, i0, dn, u, lane, acc);
-    for (; u < nu; u += NW) bjm_fwd<NT8, true>(x0, x1, rfa, i0, dn, u, lane, acc);
+    for (; u < nfull; u += NW) bjm_fwd<NT8, PRE, false>(x0, x1, rfa, i0, dn, u, lane, acc);
+    for (; u < nu; u += NW) bjm_fwd<NT8, PRE, true>(x0, x1, rfa, i0, dn, u, lane, acc);
     {
       const int g = lane >> 2, t = lane & 3;
 #pragma unroll
@@ -347,10 +366,10 @@ __global__ void __launch_bounds__(32 * NW, NW >= 16 ? 1 : 16 / NW)
   if (tid == 0 && s_bad) atomicExch(err, 1);
 }
 
-template <int NT8, int NW, int CG>
+template <int NT8, int NW, int CG, bool PRE = true>
 static cudaError_t bjm_launch(const BjArgs &a, const float *X, const float *r, float *z, int32_t *err, cudaStream_t s) {
-  typedef BjmLayout<NT8, NW> L;
-  const void *fn = (const void *)k_bj_mma<NT8, NW, CG>;
+  typedef BjmLayout<NT8, NW, PRE> L;
+  const void *fn = (const void *)k_bj_mma<NT8, NW, CG, PRE>;
   // two stages unless one leaves room for a second CTA on the SM (or two do not fit)
   const int stages = L::bytes(a.n, 2) <= 225 * 1024 && (L::bytes(a.n, 1) > 112 * 1024 || L::bytes(a.n, 2) <= 75 * 1024)
                          ? 2
@@ -373,7 +392,7 @@ static cudaError_t bjm_launch(const BjArgs &a, const float *X, const float *r, f
   at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_bj_mma<NT8, NW, CG>, a, X, r, z, stages, cs, err);
+  return cudaLaunchKernelEx(&cfg, k_bj_mma<NT8, NW, CG, PRE>, a, X, r, z, stages, cs, err);
 }
 
 template <int NT8>
@@ -386,7 +405,13 @@ static cudaError_t bjm_by_size(const BjArgs &a, const float *X, const float *r, 
   if (a.n <= 512) return bjm_launch<NT8, 16, 1>(a, X, r, z, err, s);
   // up to 8 right-hand sides two CTAs of 8 warps share an SM
   if (NT8 == 1 && a.n <= 768) return bjm_launch<1, 8, 3>(a, X, r, z, err, s);
-  if (a.n <= 1024) return bjm_launch<NT8, 16, 2>(a, X, r, z, err, s);
-  if (a.n <= 1536) return bjm_launch<NT8, 16, 3>(a, X, r, z, err, s);
+  if (a.n <= 768) return bjm_launch<NT8, 16, 2>(a, X, r, z, err, s);
+  // 16 right-hand sides of r take twice the room in split form: beyond n = 768 they leave
+  // none for a second stage (64 blocks of 1000: 110 -> 82 us as FP32 values) or for the first
+  // one (64 of 1331: 234 us by 8 right-hand sides per CTA, 162 us so); up to 768 the split at
+  // each use costs 5 %
+  constexpr bool PRE = NT8 == 1;
+  if (a.n <= 1024) return bjm_launch<NT8, 16, 2, PRE>(a, X, r, z, err, s);
+  if (a.n <= 1536) return bjm_launch<NT8, 16, 3, PRE>(a, X, r, z, err, s);
   return cudaErrorInvalidValue;
 }

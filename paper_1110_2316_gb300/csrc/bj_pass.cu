@@ -17,8 +17,7 @@ cudaError_t bj_pass_f32(const BjArgs &a, const float *X, const float *r, float *
   if (a.n_group <= 0 || a.n_rhs <= 0) return cudaSuccess;
   if (a.n_rhs == 1) return bjp_by_size<float, 1>(a, X, r, z, err, s);
   if (a.n_rhs <= 4) return bjp_by_size<float, 4>(a, X, r, z, err, s);
-  // two n8 tiles per CTA where their r fragments fit beside one stage of X
-  if (a.n_rhs <= 8 || BjmLayout<2, 16>::bytes(a.n, 1) > 225 * 1024) return bjm_by_size<1>(a, X, r, z, err, s);
+  if (a.n_rhs <= 8) return bjm_by_size<1>(a, X, r, z, err, s);
   return bjm_by_size<2>(a, X, r, z, err, s);
 }
 #endif
