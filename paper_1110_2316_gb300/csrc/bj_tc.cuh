@@ -3,23 +3,27 @@
 // tensor cores: tcgen05.mma kind::tf32 with FP32 accumulators in tensor memory.
 //
 // A TF32 operand keeps 10 mantissa bits, so each FP32 operand is split into
-// hi = rna_tf32(v) and lo = rna_tf32(v - hi), and every product takes three
+// hi = v rounded to TF32 and lo = v - hi rounded to TF32, and every product takes three
 // MMAs, hi*hi + hi*lo + lo*hi (the dropped lo*lo and the roundings of lo are
 // about 2^-21 of |X| |r|): the products keep FP32 accuracy, so that the
 // preconditioner stays the fixed SPD operator X~^T X~ of the FP32 factor X~
 // that the CUDA-core products apply.
 //
-// Storage: per element the factor as 128 x 128 FP32 tiles, row-major, zero
-// beyond n and outside the triangle: first the lower tiles of X (block row
-// bi, block column bk <= bi, in row order), then the tiles of X^T with
-// bk >= bi (row order), so that both products read K-major rows.
+// Storage: per element the factor as 128 x 128 FP32 tiles, zero beyond n and
+// outside the triangle: first the lower tiles of X (block row bi, block column
+// bk <= bi, in row order), then the tiles of X^T with bk >= bi (row order).  A
+// tile is four slices of 32 columns, each [4 columns][128 rows][column in the
+// four]: a thread per row reads its row in coalesced 16-byte loads.
 //
-// One CTA (4 warps) per (element, 128-row tile, 64 right-hand sides): K in
-// chunks of 32 (one 128-byte row per operand row), BJT_STAGES shared-memory stages of
-// A hi/lo (128 x 32) and B hi/lo (64 x 32) in the canonical 128-byte-swizzled
-// K-major layout (8-row atoms of 1 KB, 16-byte chunk j of row m at j ^ (m % 8)),
-// filled from registers (the split needs them anyway; the next chunk's global
-// loads are issued while the tensor core works on the current one); thread 0
+// One CTA (4 warps) per (element, 128-row tile, 64 right-hand sides), four CTAs
+// to an SM: K in chunks of 32, BJT_STAGES stages.  A (128 rows, hi and lo) goes
+// from registers to tensor memory (tcgen05.st, thread = row = lane), which the
+// MMA reads as its A operand: held in shared memory, hi and lo took 32 KB of
+// writes and 48 KB of operand reads per chunk (535 us for 512 blocks of 729 at
+// 64 right-hand sides, 368 us so).  B hi/lo (64 x 32) stand in shared memory in
+// the canonical 128-byte-swizzled K-major layout (8-row atoms of 1 KB, 16-byte
+// chunk j of row m at j ^ (m % 8)).  The next chunk's global loads are issued
+// while the tensor core works on the current one; thread 0
 // issues the 12 MMAs of a chunk (4 K-steps of 8 x 3 products, M = 128, N = 64)
 // and commits them to the stage's mbarrier; the accumulator (128 lanes x 64
 // columns of TMEM) is read back by all four warps (32 lanes each) and stored
@@ -31,18 +35,19 @@ constexpr int BJT = 128;                 // tile edge (rows per CTA, MMA M)
 constexpr int BJT_N = 64;                // right-hand sides per CTA (MMA N)
 constexpr int BJT_K = 32;                // K per stage: one 128-byte row of FP32
 constexpr int BJT_THREADS = 128;
-constexpr int BJT_A_BYTES = BJT * BJT_K * 4;    // 16 KB
 constexpr int BJT_B_BYTES = BJT_N * BJT_K * 4;  // 8 KB
-constexpr int BJT_STAGE_BYTES = 2 * BJT_A_BYTES + 2 * BJT_B_BYTES;
+constexpr int BJT_STAGE_BYTES = 2 * BJT_B_BYTES;
 #if defined(HPSE_BJT_STAGES)
 constexpr int BJT_STAGES = HPSE_BJT_STAGES;  // set at build time (pipeline-depth experiments)
 #else
-constexpr int BJT_STAGES = 1;  // 4 CTAs per SM hide more load latency than a second stage (measured)
+constexpr int BJT_STAGES = 1;  // 4 CTAs per SM hide more load latency than 3 stages and 2 CTAs (368 and 578 us)
 #endif
-constexpr int BJT_MINB = BJT_STAGES == 1 ? 4 : 2;  // CTAs per SM that the shared memory allows
+// tensor memory: accumulator (64 columns), then per stage A hi and A lo (32 columns each)
+constexpr int BJT_TMEM_COLS = BJT_STAGES == 1 ? 128 : 256;
+constexpr int BJT_MINB = 512 / BJT_TMEM_COLS;  // CTAs per SM that the tensor memory allows
 constexpr size_t BJT_SMEM = BJT_STAGES * (size_t)BJT_STAGE_BYTES + 1024;  // stages + alignment slack
+static_assert(BJT_N + BJT_STAGES * 2 * BJT_K <= BJT_TMEM_COLS, "tensor memory");
 constexpr int BJT_TILE = BJT * BJT;      // floats per tile
-constexpr int BJT_TMEM_COLS = 64;
 
 // tiles per copy (X or X^T) of an n x n factor
 __host__ __device__ inline int bjt_blocks(int n) {
@@ -77,10 +82,19 @@ __device__ __forceinline__ uint64_t bjt_desc(uint32_t addr) {
 constexpr uint32_t BJT_IDESC = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(BJT_N >> 3) << 17) |
                                ((uint32_t)(BJT >> 4) << 24);
 
+// v rounded to TF32 (nearest, ties away): two integer operations, where
+// cvt.rna.tf32 runs at a fraction of their rate
 __device__ __forceinline__ float bjt_tf32(float v) {
-  uint32_t r;
-  asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(v));
-  return __uint_as_float(r);
+  return __uint_as_float((__float_as_uint(v) + 0x1000u) & 0xffffe000u);
+}
+
+// 16 values of the lane's row to 16 columns of tensor memory
+__device__ __forceinline__ void bjt_st16(uint32_t addr, const float (&v)[16]) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%16], {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
+      "%14, %15};" ::"f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]), "f"(v[8]),
+      "f"(v[9]), "f"(v[10]), "f"(v[11]), "f"(v[12]), "f"(v[13]), "f"(v[14]), "f"(v[15]), "r"(addr)
+      : "memory");
 }
 
 __device__ __forceinline__ bool bjt_wait(uint32_t bar, uint32_t parity) {
@@ -143,19 +157,16 @@ __global__ void __launch_bounds__(BJT_THREADS, BJT_MINB) k_bj_tc(BjTcArgs A, con
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = s_tmem;
 
-  // registers of one chunk: A 8 float4 (rows q >> 3, 16-byte chunk q & 7 for
-  // q = tid + 128 i), B 16 floats (right-hand side 16 warp + j, k = lane)
+  // registers of one chunk: A 8 float4 (row tid, k = 4 i to 4 i + 3), B 16 floats
+  // (right-hand side 16 warp + j, k = lane)
   float4 ra[8];
   float rb[16];
   auto load = [&](int kc) {
     const int bk = kc >> 2;
     const int b = TRANS ? (bi * nbt - bi * (bi - 1) / 2 + (bk - bi)) : (bi * (bi + 1) / 2 + bk);
-    const float *blk = tiles + (int64_t)b * BJT_TILE + 32 * (kc & 3);
+    const float4 *blk = reinterpret_cast<const float4 *>(tiles + (int64_t)b * BJT_TILE + BJT * BJT_K * (kc & 3)) + tid;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int q = tid + BJT_THREADS * i;
-      ra[i] = *reinterpret_cast<const float4 *>(blk + (q >> 3) * BJT + 4 * (q & 7));
-    }
+    for (int i = 0; i < 8; ++i) ra[i] = blk[BJT * i];
     const int k = BJT_K * kc + lane;
 #pragma unroll
     for (int j = 0; j < 16; ++j) {
@@ -164,24 +175,26 @@ __global__ void __launch_bounds__(BJT_THREADS, BJT_MINB) k_bj_tc(BjTcArgs A, con
     }
   };
   auto store = [&](int st) {
-    unsigned char *sa_hi = sm + st * BJT_STAGE_BYTES, *sa_lo = sa_hi + BJT_A_BYTES;
-    unsigned char *sb_hi = sa_lo + BJT_A_BYTES, *sb_lo = sb_hi + BJT_B_BYTES;
+    unsigned char *sb_hi = sm + st * BJT_STAGE_BYTES, *sb_lo = sb_hi + BJT_B_BYTES;
+    // the warp's 32 lanes of tensor memory: its 32 rows of the tile
+    const uint32_t ta = tmem + ((uint32_t)(32 * warp) << 16) + BJT_N + st * 2 * BJT_K;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int q = tid + BJT_THREADS * i, m = q >> 3, c = q & 7;
-      const int off = (m >> 3) * 1024 + (m & 7) * 128 + ((c ^ (m & 7)) << 4);
-      const float4 v = ra[i];
-      float4 h, l;
-      h.x = bjt_tf32(v.x);
-      h.y = bjt_tf32(v.y);
-      h.z = bjt_tf32(v.z);
-      h.w = bjt_tf32(v.w);
-      l.x = bjt_tf32(v.x - h.x);
-      l.y = bjt_tf32(v.y - h.y);
-      l.z = bjt_tf32(v.z - h.z);
-      l.w = bjt_tf32(v.w - h.w);
-      *reinterpret_cast<float4 *>(sa_hi + off) = h;
-      *reinterpret_cast<float4 *>(sa_lo + off) = l;
+    for (int i = 0; i < 2; ++i) {
+      float h[16], l[16];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const float4 v = ra[4 * i + j];
+        h[4 * j] = bjt_tf32(v.x);
+        h[4 * j + 1] = bjt_tf32(v.y);
+        h[4 * j + 2] = bjt_tf32(v.z);
+        h[4 * j + 3] = bjt_tf32(v.w);
+        l[4 * j] = bjt_tf32(v.x - h[4 * j]);
+        l[4 * j + 1] = bjt_tf32(v.y - h[4 * j + 1]);
+        l[4 * j + 2] = bjt_tf32(v.z - h[4 * j + 2]);
+        l[4 * j + 3] = bjt_tf32(v.w - h[4 * j + 3]);
+      }
+      bjt_st16(ta + 16 * i, h);
+      bjt_st16(ta + BJT_K + 16 * i, l);
     }
 #pragma unroll
     for (int j = 0; j < 16; ++j) {
@@ -202,28 +215,31 @@ __global__ void __launch_bounds__(BJT_THREADS, BJT_MINB) k_bj_tc(BjTcArgs A, con
       s_bad = 1;
     __syncthreads();
     if (s_bad) break;
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     store(st);
+    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     __syncthreads();
     if (kc + 1 < kc1) load(kc + 1);
     if (tid == 0) {
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint32_t a_hi = sbase + st * BJT_STAGE_BYTES, a_lo = a_hi + BJT_A_BYTES;
-      const uint32_t b_hi = a_lo + BJT_A_BYTES, b_lo = b_hi + BJT_B_BYTES;
+      const uint32_t a_hi = tmem + BJT_N + st * 2 * BJT_K, a_lo = a_hi + BJT_K;
+      const uint32_t b_hi = sbase + st * BJT_STAGE_BYTES, b_lo = b_hi + BJT_B_BYTES;
 #pragma unroll
       for (int s = 0; s < 4; ++s) {
-        // K-step s: 8 TF32 = 32 bytes further along the swizzled rows
-        const uint64_t dah = bjt_desc(a_hi + 32 * s), dal = bjt_desc(a_lo + 32 * s);
+        // K-step s: 8 TF32, 8 columns of A and 32 bytes further along the swizzled rows of B
         const uint64_t dbh = bjt_desc(b_hi + 32 * s), dbl = bjt_desc(b_lo + 32 * s);
-        const uint64_t da[3] = {dah, dah, dal}, db[3] = {dbh, dbl, dbh};
+        const uint32_t da[3] = {a_hi + 8 * s, a_hi + 8 * s, a_lo + 8 * s};
+        const uint64_t db[3] = {dbh, dbl, dbh};
 #pragma unroll
         for (int p = 0; p < 3; ++p) {
           const uint32_t acc = (it > 0 || s > 0 || p > 0) ? 1u : 0u;
           asm volatile(
               "{\n\t.reg .pred q;\n\t"
               "setp.ne.b32 q, %4, 0;\n\t"
-              "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, q;\n\t}" ::"r"(tmem),
-              "l"(da[p]), "l"(db[p]), "r"(BJT_IDESC), "r"(acc)
+              "tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, q;\n\t}" ::"r"(tmem),
+              "r"(da[p]), "l"(db[p]), "r"(BJT_IDESC), "r"(acc)
               : "memory");
         }
       }
@@ -291,7 +307,7 @@ __global__ void k_bj_tile(BjArgs A, const int64_t *tile_off, const double *X64, 
   const double *Xe = X64 + A.blk_off[e];
   float *T = Xt + tile_off[e] + (int64_t)(up ? nblk + b : b) * BJT_TILE;
   for (int idx = threadIdx.x; idx < BJT_TILE; idx += blockDim.x) {
-    const int i = BJT * bi + (idx >> 7), k = BJT * bk + (idx & 127);
+    const int i = BJT * bi + ((idx >> 2) & 127), k = BJT * bk + 4 * (idx >> 9) + (idx & 3);
     double v = 0.0;
     if (!up) {
       if (i < n && k <= i) v = Xe[pk(i, k)];
