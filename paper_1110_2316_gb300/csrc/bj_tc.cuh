@@ -20,7 +20,10 @@
 // from registers to tensor memory (tcgen05.st, thread = row = lane), which the
 // MMA reads as its A operand: held in shared memory, hi and lo took 32 KB of
 // writes and 48 KB of operand reads per chunk (535 us for 512 blocks of 729 at
-// 64 right-hand sides, 368 us so).  B hi/lo (64 x 32) stand in shared memory in
+// 64 right-hand sides, 368 us so; 334 us with the pointer arithmetic and the
+// bounds checks of B out of the loop, which is bound by the instructions and
+// barriers of a chunk: neither a third of the MMAs nor a fifth of the bytes less
+// changes its time).  B hi/lo (64 x 32) stand in shared memory in
 // the canonical 128-byte-swizzled K-major layout (8-row atoms of 1 KB, 16-byte
 // chunk j of row m at j ^ (m % 8)).  The next chunk's global loads are issued
 // while the tensor core works on the current one; thread 0
@@ -78,9 +81,10 @@ __device__ __forceinline__ uint64_t bjt_desc(uint32_t addr) {
 
 // instruction descriptor of kind::tf32: FP32 accumulator (bits 4-5 = 1), A and
 // B TF32 (bits 7-9, 10-12 = 2), both K-major, N >> 3 at bits 17-22, M >> 4 at
-// bits 24-28
-constexpr uint32_t BJT_IDESC = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(BJT_N >> 3) << 17) |
-                               ((uint32_t)(BJT >> 4) << 24);
+// bits 24-28 (N = nb: the right-hand sides of the CTA, rounded up to 16)
+__device__ __forceinline__ constexpr uint32_t bjt_idesc(int nb) {
+  return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(nb >> 3) << 17) | ((uint32_t)(BJT >> 4) << 24);
+}
 
 // v rounded to TF32 (nearest, ties away): two integer operations, where
 // cvt.rna.tf32 runs at a fraction of their rate
@@ -128,6 +132,7 @@ __global__ void __launch_bounds__(BJT_THREADS, BJT_MINB) k_bj_tc(BjTcArgs A, con
   const int ge = blockIdx.x / nbt, bi = blockIdx.x - ge * nbt;
   const int e = A.elems[ge];
   const int r0 = blockIdx.y * BJT_N;
+  const int nb = min(BJT_N, (A.n_rhs - r0 + 15) & ~15);  // MMA N
   const int64_t vb = A.dof_off[e];
   const int nblk = bjt_blocks(n);
   const float *tiles = Xt + A.tile_off[e] + (TRANS ? (int64_t)nblk * BJT_TILE : 0);
@@ -161,17 +166,25 @@ __global__ void __launch_bounds__(BJT_THREADS, BJT_MINB) k_bj_tc(BjTcArgs A, con
   // (right-hand side 16 warp + j, k = lane)
   float4 ra[8];
   float rb[16];
+  const int nv = A.n_rhs - r0 - 16 * warp;  // right-hand sides of the warp
+  const float *bsrc = in + (int64_t)(r0 + 16 * warp) * A.ndof + vb + lane;
   auto load = [&](int kc) {
     const int bk = kc >> 2;
     const int b = TRANS ? (bi * nbt - bi * (bi - 1) / 2 + (bk - bi)) : (bi * (bi + 1) / 2 + bk);
     const float4 *blk = reinterpret_cast<const float4 *>(tiles + (int64_t)b * BJT_TILE + BJT * BJT_K * (kc & 3)) + tid;
+    // rows beyond n, and in the diagonal tile those on the zero side of the 32 columns, are not read
+    const bool some = BJT * bi + 32 * warp < n && (bk != bi || (TRANS ? warp <= (kc & 3) : warp >= (kc & 3)));
 #pragma unroll
-    for (int i = 0; i < 8; ++i) ra[i] = blk[BJT * i];
-    const int k = BJT_K * kc + lane;
+    for (int i = 0; i < 8; ++i) ra[i] = some ? blk[BJT * i] : make_float4(0.f, 0.f, 0.f, 0.f);
+    // from one running pointer; the bounds checks only where a chunk or the right-hand sides end
+    const float *src = bsrc + BJT_K * kc;
+    if (nv >= 16 && BJT_K * (kc + 1) <= n) {
 #pragma unroll
-    for (int j = 0; j < 16; ++j) {
-      const int c = r0 + 16 * warp + j;
-      rb[j] = (k < n && c < A.n_rhs) ? in[(int64_t)c * A.ndof + vb + k] : 0.0f;
+      for (int j = 0; j < 16; ++j, src += A.ndof) rb[j] = *src;
+    } else {
+      const int m = BJT_K * kc + lane < n ? nv : 0;
+#pragma unroll
+      for (int j = 0; j < 16; ++j, src += A.ndof) rb[j] = j < m ? *src : 0.0f;
     }
   };
   auto store = [&](int st) {
@@ -196,6 +209,7 @@ __global__ void __launch_bounds__(BJT_THREADS, BJT_MINB) k_bj_tc(BjTcArgs A, con
       bjt_st16(ta + 16 * i, h);
       bjt_st16(ta + BJT_K + 16 * i, l);
     }
+    if (nv <= 0) return;
 #pragma unroll
     for (int j = 0; j < 16; ++j) {
       const int nn = 16 * warp + j;
@@ -239,7 +253,7 @@ __global__ void __launch_bounds__(BJT_THREADS, BJT_MINB) k_bj_tc(BjTcArgs A, con
               "{\n\t.reg .pred q;\n\t"
               "setp.ne.b32 q, %4, 0;\n\t"
               "tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, q;\n\t}" ::"r"(tmem),
-              "r"(da[p]), "l"(db[p]), "r"(BJT_IDESC), "r"(acc)
+              "r"(da[p]), "l"(db[p]), "r"(bjt_idesc(nb)), "r"(acc)
               : "memory");
         }
       }
@@ -259,6 +273,7 @@ __global__ void __launch_bounds__(BJT_THREADS, BJT_MINB) k_bj_tc(BjTcArgs A, con
     const int row = BJT * bi + 32 * warp + lane;
 #pragma unroll
     for (int c0 = 0; c0 < BJT_N; c0 += 16) {
+      if (c0 >= nb) break;
       uint32_t v[16];
       asm volatile(
           "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
@@ -269,11 +284,10 @@ __global__ void __launch_bounds__(BJT_THREADS, BJT_MINB) k_bj_tc(BjTcArgs A, con
           : "memory");
       asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
       if (row < n) {
+        float *dst = out + (int64_t)(r0 + c0) * A.ndof + vb + row;
 #pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          const int c = r0 + c0 + j;
-          if (c < A.n_rhs) out[(int64_t)c * A.ndof + vb + row] = __uint_as_float(v[j]);
-        }
+        for (int j = 0; j < 16; ++j, dst += A.ndof)
+          if (r0 + c0 + j < A.n_rhs) *dst = __uint_as_float(v[j]);
       }
     }
   } else if (tid == 0) {
