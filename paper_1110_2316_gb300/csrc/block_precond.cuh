@@ -379,7 +379,7 @@ __global__ void __launch_bounds__(TR *TC) k_bj_tri(BjArgs A, const T *X, const T
 // Vector kernels of the PCG step, one warp per (element, rhs) item, eight items
 // per CTA: the FP64 sums are bound by the FP64 pipe, and a warp that keeps its
 // item's whole sum adds five values in the end, where a CTA per item added five
-// per warp (config 2, 16 rhs: 46 + 48 us for the pair, HBM 21 + 7).
+// per warp (512 blocks of 729, 16 rhs: 46 + 48 us for the pair, HBM 21 + 7).
 constexpr int BJ_VEC_ITEMS = 8;
 inline unsigned bj_vec_grid(int items) { return (unsigned)((items + BJ_VEC_ITEMS - 1) / BJ_VEC_ITEMS); }
 
@@ -429,8 +429,8 @@ __global__ void __launch_bounds__(32 * BJ_VEC_ITEMS) k_bj_dot(BjArgs A, const T 
 // (rows x right-hand sides per CTA), variant 8 is the tensor-core form
 // (bj_tc.cuh: 128 rows x 64 right-hand sides, 3xTF32), offered from 32
 // right-hand sides on.  Variants 2, 4, 6 and 8 exist in FP32 only.
-// Config 2's factors (512 blocks of 729), one application, tiles -> pass:
-// FP32 270 -> 145 us (1 rhs), 468 -> 215 (4), 470 -> 242 (8), 871 -> 365 (16);
+// 512 factors of n = 729, one application, tiles -> pass:
+// FP32 270 -> 145 us (1 rhs), 468 -> 215 (4), 470 -> 242 (8), 871 -> 359 (16);
 // FP64 4820 -> 2417 us (4), 4810 -> 4600 (8), and for 8 blocks 400 -> 98 us
 // (4).  One FP64 right-hand side of many blocks stays with the 64 x 1 tile
 // (622 us against 767), of few blocks the pass is the faster (41 against 89).

@@ -844,7 +844,7 @@ __device__ __forceinline__ FaceMeta *face_meta(real *stab) {
 // every T access of both y-stages, a third of the FP32 kernel's shared
 // wavefronts); FP32 rows are padded to a stride of Q mod 32, which makes a
 // warp's addresses distinct, where the padding costs no resident CTA
-// (config 2's apply 418 -> 410 us at 16 rhs, W = 7 306 -> 288 us).
+// (512 elements and 16 rhs: W = 8 418 -> 410 us, W = 7 306 -> 288 us).
 constexpr int T_PAD = sizeof(real) == 4 ? (((Q - Q2) % 32) + 32) % 32 : 0;
 // the FP64 reduction of PCG's p.q uses the X fields, free by then, where they
 // hold NT doubles, else NT doubles after everything else
