@@ -4,8 +4,9 @@
 // preconditioner (Section 5.2, eq. 5.19-5.20, which is kept as the default);
 // a block-Jacobi alternative on the same element blocks.
 //
-// Set-up (FP64): A_ee is probed column by column with the operator kernel in
-// self-only mode (neighbour traces taken as zero), gathered into packed
+// Set-up (FP64): A_ee is formed column by column with the operator kernel in
+// self-only mode (neighbour traces taken as zero; MODE_PROBE, or MODE_PLAIN on
+// unit vectors for the general, curved and neighbourhood operators), gathered into packed
 // lower-triangular storage (row i holds columns 0..i at offset i(i+1)/2),
 // factored A_ee = L L^T and X = L^{-1} is formed, both in 64 x 64 tiles.  The preconditioner is z = X^T (X r): two
 // triangular products, kept in FP64 and rounded to FP32.  Storing the factor

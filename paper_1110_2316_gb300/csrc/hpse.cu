@@ -2975,14 +2975,20 @@ extern "C" hpse_status hpse_setup_block_preconditioner(hpse_mesh *m) {
     a.n_rhs = nc;
     a.self_only = 1;
     const int th = m->threads[0][0][g.W];
+    // unit vectors through memory only where another kernel reads them
+    const bool unit = !(m->apply_coef == hpse::COEF_LAPLACE || m->apply_coef == hpse::COEF_SCALAR);
     for (int j0 = 0; j0 < n; j0 += nc) {
       const int c = std::min(nc, n - j0);
       const KernelSet &ks = apply_set(m, 0, g.W, (long long)g.n * c, (long long)g.n * c);
       a.n_rhs = c;
       ba.n_rhs = c;
-      k_bj_probe<<<g.n * c, 128, 0, s>>>(ba, j0, c, pu.as<double>());
-      CK(cudaGetLastError());
-      CK(ks.apply(m->apply_coef, MODE_PLAIN, &a, g.n * c, th, s));
+      a.probe0 = j0;
+      if (unit || m->has_mixed || m->curved) {
+        k_bj_probe<<<g.n * c, 128, 0, s>>>(ba, j0, c, pu.as<double>());
+        CK(cudaGetLastError());
+        ++g_launches;
+      }
+      CK(ks.apply(m->apply_coef, unit ? MODE_PLAIN : hpse::MODE_PROBE, &a, g.n * c, th, s));
       {
         hpse_status st = launch_mixed<double>(m, MODE_PLAIN, pu.as<double>(), py.as<double>(), nullptr, c, 1, g.W, s);
         if (st != HPSE_OK) return st;
@@ -2991,7 +2997,7 @@ extern "C" hpse_status hpse_setup_block_preconditioner(hpse_mesh *m) {
       }
       k_bj_gather<<<g.n * c, 128, 0, s>>>(ba, j0, c, py.as<double>(), blk.as<double>());
       CK(cudaGetLastError());
-      g_launches += 3;
+      g_launches += 2;
     }
     // A = L L^T, X = L^{-1} by 64 x 64 tiles
     const int nb = (n + BJB - 1) / BJB;

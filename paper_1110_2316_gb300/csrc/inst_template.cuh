@@ -26,11 +26,17 @@ cudaError_t apply_fn(int coef, int mode, const void *args, int n_items, int thre
     if (mode == MODE_PCG) return launch_apply_t<COEF_LAPLACE, MODE_PCG>(args, n_items, threads, s);
     if (mode == MODE_TRANSPOSE) return launch_apply_t<COEF_LAPLACE, MODE_TRANSPOSE>(args, n_items, threads, s);
     if (mode == MODE_RESIDUAL) return launch_apply_t<COEF_LAPLACE, MODE_RESIDUAL>(args, n_items, threads, s);
+#if defined(HPSE_DOUBLE)
+    if (mode == MODE_PROBE) return launch_apply_t<COEF_LAPLACE, MODE_PROBE>(args, n_items, threads, s);
+#endif
   } else if (coef == COEF_SCALAR) {
     if (mode == MODE_PLAIN) return launch_apply_t<COEF_SCALAR, MODE_PLAIN>(args, n_items, threads, s);
     if (mode == MODE_PCG) return launch_apply_t<COEF_SCALAR, MODE_PCG>(args, n_items, threads, s);
     if (mode == MODE_TRANSPOSE) return launch_apply_t<COEF_SCALAR, MODE_TRANSPOSE>(args, n_items, threads, s);
     if (mode == MODE_RESIDUAL) return launch_apply_t<COEF_SCALAR, MODE_RESIDUAL>(args, n_items, threads, s);
+#if defined(HPSE_DOUBLE)
+    if (mode == MODE_PROBE) return launch_apply_t<COEF_SCALAR, MODE_PROBE>(args, n_items, threads, s);
+#endif
   } else if (coef == COEF_EDGE) {
     if (mode == MODE_PLAIN) return launch_apply_t<COEF_EDGE, MODE_PLAIN>(args, n_items, threads, s);
     if (mode == MODE_PCG) return launch_apply_t<COEF_EDGE, MODE_PCG>(args, n_items, threads, s);
@@ -196,6 +202,10 @@ cudaError_t upload_fn(const double *pk) {
   if ((e2 = set_smem_attr<COEF_SCALAR, MODE_PCG>()) != cudaSuccess) return e2;
   if ((e2 = set_smem_attr<COEF_SCALAR, MODE_TRANSPOSE>()) != cudaSuccess) return e2;
   if ((e2 = set_smem_attr<COEF_SCALAR, MODE_RESIDUAL>()) != cudaSuccess) return e2;
+#if defined(HPSE_DOUBLE)
+  if ((e2 = set_smem_attr<COEF_LAPLACE, MODE_PROBE>()) != cudaSuccess) return e2;
+  if ((e2 = set_smem_attr<COEF_SCALAR, MODE_PROBE>()) != cudaSuccess) return e2;
+#endif
   if ((e2 = set_smem_attr<COEF_EDGE, MODE_PLAIN>()) != cudaSuccess) return e2;
   if ((e2 = set_smem_attr<COEF_EDGE, MODE_PCG>()) != cudaSuccess) return e2;
   if ((e2 = set_smem_attr<COEF_EDGE, MODE_TRANSPOSE>()) != cudaSuccess) return e2;

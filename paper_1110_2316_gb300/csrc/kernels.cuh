@@ -158,6 +158,7 @@ using hpse::MODE_PLAIN;
 using hpse::MODE_PCG;
 using hpse::MODE_TRANSPOSE;
 using hpse::MODE_RESIDUAL;
+using hpse::MODE_PROBE;
 typedef hpse::ApplyArgsT<real> ApplyArgs;
 typedef hpse::PrecArgsT<real> PrecArgs;
 
@@ -1341,8 +1342,18 @@ __global__ void __launch_bounds__(NT, APPLY_MINB) k_apply(const ApplyArgs A) {
 
   for (int t = tid; t < P2; t += nt) stab[t] = c_tab.D[t];
   FaceMeta *fm = face_meta(stab);
-  if ((MODE == MODE_PLAIN || MODE == MODE_PCG) && tid < 6) face_meta_fill<COEF, MODE>(A, e, r, geo_e, fm, tid);
-  if (MODE != MODE_TRANSPOSE) {
+  if ((MODE == MODE_PLAIN || MODE == MODE_PCG || MODE == MODE_PROBE) && tid < 6)
+    face_meta_fill<COEF, MODE>(A, e, r, geo_e, fm, tid);
+  // MODE_PROBE: u is the unit vector of node (ju, jv, jw), so that every field of the
+  // forward stages is a product of three table entries, formed where the z-stage uses it;
+  // only the nodes from plane jw on are transposed (the rows at and below the diagonal):
+  // the set-up of 64 element blocks of W = 8, bound by the FP64 pipe in these columns,
+  // 93.5 -> 68.3 ms against MODE_PLAIN on unit vectors
+  const int ju = MODE == MODE_PROBE ? (A.probe0 + r) % P : 0, jv = MODE == MODE_PROBE ? (A.probe0 + r) / P % P : 0;
+  const int jw = MODE == MODE_PROBE ? (A.probe0 + r) / P2 : 0;
+  if (MODE == MODE_PROBE) {
+    for (int t = tid; t < P3; t += nt) su[t] = t == A.probe0 + r ? (real)1 : (real)0;
+  } else if (MODE != MODE_TRANSPOSE) {
     if (MODE == MODE_PCG) {
       const double bt = A.beta[A.prob[e] * A.n_rhs + r];
       for (int t = tid; t < P3; t += nt) {
@@ -1489,6 +1500,24 @@ __global__ void __launch_bounds__(NT, APPLY_MINB) k_apply(const ApplyArgs A) {
       } else {
 #pragma unroll
         for (int qc = 0; qc < Q; ++qc) rho[qc] = (real)A.rho[(int64_t)r * A.nquad + cbase + (int64_t)qc * Q2];
+      }
+      __syncwarp();  // lanes past the last column read its rho
+    } else if constexpr (MODE == MODE_PROBE) {
+      const real x0 = c_tab.B[0][qa * P + ju], x1 = c_tab.B[1][qa * P + ju], x2 = c_tab.B[2][qa * P + ju];
+      const real y0 = c_tab.B[0][qb * P + jv], y1 = c_tab.B[1][qb * P + jv], y2 = c_tab.B[2][qb * P + jv];
+      const real t00 = x0 * y0, tl = sx2 * (x2 * y0) + sy2 * (x0 * y2), t10 = x1 * y0, t01 = x0 * y1;
+      const real wab = c_tab.WQ[qa] * c_tab.WQ[qb] * Jac;
+#pragma unroll
+      for (int q = 0; q < Q; ++q) {
+        const real z0 = c_tab.B[0][q * P + jw], z1 = c_tab.B[1][q * P + jw], z2 = c_tab.B[2][q * P + jw];
+        const real sigma0 = sz2c * z2 * t00 + z0 * tl;
+        if (var_coef(COEF)) {
+          real mq, dx, dy, dz;
+          load_coef4(A.coef + 4 * (cbase + (int64_t)q * Q2), mq, dx, dy, dz);
+          rho[q] = mq * (sigma0 + dz * (z1 * t00) + z0 * (dx * t10 + dy * t01));
+        } else {
+          rho[q] = wab * c_tab.WQ[q] * sigma0;
+        }
       }
       __syncwarp();  // lanes past the last column read its rho
     } else if constexpr (packed_coef(COEF, 4)) {
@@ -1720,6 +1749,7 @@ __global__ void __launch_bounds__(NT, APPLY_MINB) k_apply(const ApplyArgs A) {
       const bool ok = lp < QP;
       const int l = ok ? lp : QP - 1;
       const int qa = l % Q, k = l / Q;
+      if (MODE == MODE_PROBE && __all_sync(0xffffffffu, k < jw)) continue;
       const real sy2q = (COEF == COEF_VERTEX) ? sy2 * A.kappa[(int64_t)e * hpse::KAPPA_STRIDE + qa] : sy2;
       const real sx2q =
           (COEF == COEF_VERTEX_EDGE) ? sx2 * ((real)1 + A.kappa[(int64_t)e * hpse::KAPPA_STRIDE + qa]) : sx2;
@@ -1746,6 +1776,7 @@ __global__ void __launch_bounds__(NT, APPLY_MINB) k_apply(const ApplyArgs A) {
       const int c = it / LS::PADL, lp = it - c * LS::PADL;
       const bool ok = lp < P2;
       const int l = ok ? lp : P2 - 1;
+      if (MODE == MODE_PROBE && __all_sync(0xffffffffu, l / P < jw)) continue;
       if constexpr (packed_coef(COEF, 32) && packed_mode(COEF, MODE)) {
 #define XR_CALL(CI) x_rev_chunk2<COEF, (CI < LS::NC ? CI : 0), LS::NC>(X0, X1, X2, sy, l, ok)
         HPSE_DISPATCH4(LS::NC, c, XR_CALL);

@@ -43,7 +43,9 @@ enum { COEF_LAPLACE = 0, COEF_SCALAR = 1, COEF_EDGE = 2, COEF_VERTEX = 3, COEF_V
 // KAPPA_STRIDE = 2 * HPSE_MAX_W + 1, CSCR_STRIDE = HPSE_MAX_W + 1 (checked in the host library)
 enum { KAPPA_STRIDE = 21, CSCR_STRIDE = 11, FACE_W = 10, ZEIG_STRIDE = 132 };
 // MODE_RESIDUAL: z = sqrt(w J) (L u - f) at the volume points, no transpose (COEF_LAPLACE, COEF_SCALAR)
-enum { MODE_PLAIN = 0, MODE_PCG = 1, MODE_TRANSPOSE = 2, MODE_RESIDUAL = 3 };
+// MODE_PROBE: column probe0 + (the item's right-hand side) of the element's diagonal block
+// A_ee (FP64, COEF_LAPLACE, COEF_SCALAR; with self_only), rows at and below the diagonal
+enum { MODE_PLAIN = 0, MODE_PCG = 1, MODE_TRANSPOSE = 2, MODE_RESIDUAL = 3, MODE_PROBE = 4 };
 
 template <typename T>
 struct ApplyArgsT {
@@ -75,6 +77,7 @@ struct ApplyArgsT {
   const T *zin;
   int32_t skip_faces;
   int32_t self_only;        // 1: neighbour traces taken as zero (diagonal blocks of A)
+  int32_t probe0;           // MODE_PROBE: the first column of the launch
   // edge neighbourhood (COEF_EDGE); null / 0 for box meshes
   int32_t n_elem;           // corner set c's values start at dof_off[n_elem + c]
   const T *kappa;           // [E][KAPPA_STRIDE]: per x-point factor (e^{2 tau}, 1/sin^2 phi, e^{2 psi})
