@@ -1,5 +1,5 @@
 // bj_mma.cuh -- the one-pass product z = X^T (X r) (bj_pass.cuh) for 5 to 31
-// FP32 right-hand sides: the same walk over blocks of 16 rows of X, with the
+// FP32 right-hand sides of blocks above n = 64: the same walk over blocks of 16 rows of X, with the
 // products on mma.sync m16n8k8 (TF32).  At 8 and 16 right-hand sides the packed
 // FMAs and their shared loads bound the pass (271 and 480 us for 512 blocks of
 // 729); the matrix instructions cut the issued instructions, so that what is
@@ -11,8 +11,8 @@
 // FP32 accuracy: every operand is split, v = hi + lo (TF32 each), and a product
 // takes lo hi + hi lo + hi hi.  The tensor core truncates its accumulator, so
 // sums run over 16 terms only and are added up in FP32 registers: the error
-// against 64 bits is that of the FP32 tiles (2e-7 at n = 729), where one long
-// accumulation would lose a digit.
+// against 64 bits is 1.6e-7 at n = 729 (a chain of FP32 FMAs: 4.5e-7), where one
+// long accumulation on the tensor core would lose a digit.
 //
 // Layout: the columns of a lane are chosen so that the packed rows need no
 // padding: consecutive triangular numbers are distinct modulo 2^k, so lanes on
@@ -397,8 +397,6 @@ static cudaError_t bjm_launch(const BjArgs &a, const float *X, const float *r, f
 
 template <int NT8>
 static cudaError_t bjm_by_size(const BjArgs &a, const float *X, const float *r, float *z, int32_t *err, cudaStream_t s) {
-  if (a.n <= 32) return bjm_launch<NT8, 1, 1>(a, X, r, z, err, s);
-  if (a.n <= 64) return bjm_launch<NT8, 2, 1>(a, X, r, z, err, s);
   if (a.n <= 128) return bjm_launch<NT8, 4, 1>(a, X, r, z, err, s);
   if (a.n <= 256) return bjm_launch<NT8, 4, 2>(a, X, r, z, err, s);
   if (a.n <= 384) return bjm_launch<NT8, 8, 2>(a, X, r, z, err, s);

@@ -16,7 +16,11 @@ cudaError_t bj_pass_f64(const BjArgs &a, const double *X, const double *r, doubl
 cudaError_t bj_pass_f32(const BjArgs &a, const float *X, const float *r, float *z, int32_t *err, cudaStream_t s) {
   if (a.n_group <= 0 || a.n_rhs <= 0) return cudaSuccess;
   if (a.n_rhs == 1) return bjp_by_size<float, 1>(a, X, r, z, err, s);
-  if (a.n_rhs <= 4) return bjp_by_size<float, 4>(a, X, r, z, err, s);
+  // blocks up to n = 64 keep FP32 FMAs for any count: their sums are short, and the split of
+  // the matrix instructions would be the larger error (against 64 bits, n = 8, 27, 64: 1.2e-7,
+  // 1.3e-7, 1.46e-7 against 0.6e-7, 0.97e-7, 1.38e-7 of a chain of FMAs; n = 125: 1.5e-7 against
+  // 1.9e-7), although they would be faster on many elements (8,192 of 64, 16 rhs: 90 us, 243 here)
+  if (a.n_rhs <= 4 || a.n <= 64) return bjp_by_size<float, 4>(a, X, r, z, err, s);
   if (a.n_rhs <= 8) return bjm_by_size<1>(a, X, r, z, err, s);
   return bjm_by_size<2>(a, X, r, z, err, s);
 }
