@@ -21,9 +21,9 @@
 // MMA reads as its A operand: held in shared memory, hi and lo took 32 KB of
 // writes and 48 KB of operand reads per chunk (535 us for 512 blocks of 729 at
 // 64 right-hand sides, 368 us so; 334 us with the pointer arithmetic and the
-// bounds checks of B out of the loop, which is bound by the instructions and
-// barriers of a chunk: neither a third of the MMAs nor a fifth of the bytes less
-// changes its time).  B hi/lo (64 x 32) stand in shared memory in
+// bounds checks of B out of the loop, which is bound by the latency of a
+// chunk's loads behind the barriers: neither two of three MMAs nor a fifth of the
+// bytes less changes its time).  B hi/lo (64 x 32) stand in shared memory in
 // the canonical 128-byte-swizzled K-major layout (8-row atoms of 1 KB, 16-byte
 // chunk j of row m at j ^ (m % 8)).  The next chunk's global loads are issued
 // while the tensor core works on the current one; thread 0
