@@ -87,9 +87,17 @@ __device__ __forceinline__ constexpr uint32_t bjt_idesc(int nb) {
 }
 
 // v rounded to TF32 (nearest, ties away): two integer operations, where
-// cvt.rna.tf32 runs at a fraction of their rate
+// cvt.rna.tf32 runs at a fraction of their rate.  A NaN may come out as a zero (the
+// carry of 0x7fffffff runs through the sign), so of the two parts of a split the
+// other one has to keep it.
 __device__ __forceinline__ float bjt_tf32(float v) {
   return __uint_as_float((__float_as_uint(v) + 0x1000u) & 0xffffe000u);
+}
+// the same of the rest v - hi of a right-hand side's split: NaN (0x7fffffff, what
+// the subtraction gives for v = NaN or infinity) stays NaN, so that a non-finite
+// entry reaches the product.  The factor's entries are finite and need no such care.
+__device__ __forceinline__ float bjt_tf32_rest(float v) {
+  return __int_as_float((min(__float_as_int(v), 0x7fffefff) + 0x1000) & (int)0xffffe000);
 }
 
 // 16 values of the lane's row to 16 columns of tensor memory
@@ -216,7 +224,7 @@ __global__ void __launch_bounds__(BJT_THREADS, BJT_MINB) k_bj_tc(BjTcArgs A, con
       const int off = (nn >> 3) * 1024 + (nn & 7) * 128 + ((((lane >> 2) ^ (nn & 7)) << 4) | ((lane & 3) << 2));
       const float h = bjt_tf32(rb[j]);
       *reinterpret_cast<float *>(sb_hi + off) = h;
-      *reinterpret_cast<float *>(sb_lo + off) = bjt_tf32(rb[j] - h);
+      *reinterpret_cast<float *>(sb_lo + off) = bjt_tf32_rest(rb[j] - h);
     }
   };
 
