@@ -357,6 +357,16 @@ hpse_status hpse_block_tile(const hpse_mesh *m, int32_t W, int32_t prec, int32_t
                             int32_t *tile_rhs, float *ms);
 hpse_status hpse_set_block_tile(hpse_mesh *m, int32_t W, int32_t prec, int32_t variant);
 
+/* Limit of the device waits of the block products (the one-pass and the
+ * tensor-core variants wait for copies and matrix instructions of their own): a
+ * wait gives up after `polls` polls (0 to 2^22, the default, about a second;
+ * HPSE_ERR_INVALID_ARG outside).  A product that gave up leaves NaN in its part of z; the
+ * next hpse_apply_preconditioner or hpse_pcg_solve with HPSE_PRECOND_BLOCK, and
+ * the solve in which it happened, return HPSE_ERR_CUDA until
+ * hpse_setup_block_preconditioner is called again.  The set-up drops a variant
+ * that gives up while it is timed.  Low limits are for tests of this path. */
+hpse_status hpse_set_block_wait(hpse_mesh *m, int32_t polls);
+
 /* Choose the preconditioner (hpse_precond_kind).  HPSE_PRECOND_BLOCK needs a
  * successful hpse_setup_block_preconditioner (else HPSE_ERR_NO_DATA). */
 hpse_status hpse_select_preconditioner(hpse_mesh *m, int32_t kind);

@@ -186,6 +186,10 @@ class Mesh:
     def set_block_tile(self, W, prec, variant):
         check(self._lib.hpse_set_block_tile(self._h, int(W), int(prec), int(variant)), "hpse_set_block_tile")
 
+    def set_block_wait(self, polls):
+        """Polls after which a device wait of the block products gives up (default and most: 2**22)."""
+        check(self._lib.hpse_set_block_wait(self._h, int(polls)), "hpse_set_block_wait")
+
     def select_preconditioner(self, kind):
         check(self._lib.hpse_select_preconditioner(self._h, int(kind)), "hpse_select_preconditioner")
 

@@ -150,7 +150,7 @@ __device__ __forceinline__ void bjm_back(const uint32_t (&ro)[2][2], const float
 
 template <int NT8, int NW, int CG, bool PRE>
 __global__ void __launch_bounds__(32 * NW, NW >= 16 ? 1 : 16 / NW)
-    k_bj_mma(BjArgs A, const float *X, const float *in, float *out, int stages, int cs, int32_t *err) {
+    k_bj_mma(BjArgs A, const float *X, const float *in, float *out, int stages, int cs) {
   typedef BjmLayout<NT8, NW, PRE> L;
   constexpr int RT = L::RT, NTH = 32 * NW;
   extern __shared__ __align__(16) unsigned char bjm_raw[];
@@ -277,7 +277,7 @@ __global__ void __launch_bounds__(32 * NW, NW >= 16 ? 1 : 16 / NW)
     const uint32_t Xb = block(it + 1, i0, dn, st);
     const int rg = lane >> 2, rt = lane & 3;
     const uint32_t x0 = Xb + 4 * (rg * i0 + bjp_tri(rg) + 8 * rt), x1 = Xb + 4 * ((rg + 8) * i0 + bjp_tri(rg + 8) + 8 * rt);
-    if (!bjp_wait(bjp_saddr(&bar[st]), (stages == 2 ? (it + 1) >> 1 : it + 1) & 1)) s_bad = 1;  // gives up after the barrier
+    if (!bjp_wait(bjp_saddr(&bar[st]), (stages == 2 ? (it + 1) >> 1 : it + 1) & 1, A.polls)) s_bad = 1;  // gives up after the barrier
     float acc[NT8][4];
 #pragma unroll
     for (int q = 0; q < NT8; ++q)
@@ -302,8 +302,18 @@ __global__ void __launch_bounds__(32 * NW, NW >= 16 ? 1 : 16 / NW)
     }
     __syncthreads();
     if (s_bad) {
-      // wait (bounded) for the other stage's copy before the CTA ends
-      if (stages == 2 && it + 2 < mine) bjp_wait(bjp_saddr(&bar[st ^ 1]), ((it + 2) >> 1) & 1);
+      // the copies in flight land (bounded) before their memory is used again or the CTA
+      // ends: this block's and, before the first block, the second stage's
+      bjp_wait(bjp_saddr(&bar[st]), (stages == 2 ? (it + 1) >> 1 : it + 1) & 1, BJ_POLLS);
+      if (stages == 2 && it < 0 && mine > 1) bjp_wait(bjp_saddr(&bar[1]), 0, BJ_POLLS);
+#pragma unroll
+      for (int c = 0; c < CG; ++c)
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+#pragma unroll
+          for (int q = 0; q < NT8; ++q)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) z[c][j][q][i] = __int_as_float(0x7fffffff);
       break;
     }
     if (stages == 2 && it >= 0 && it + 2 < mine && tid == 0) {
@@ -363,11 +373,11 @@ __global__ void __launch_bounds__(32 * NW, NW >= 16 ? 1 : 16 / NW)
     }
     asm volatile("barrier.cluster.arrive.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
   }
-  if (tid == 0 && s_bad) atomicExch(err, 1);
+  if (tid == 0 && s_bad) bj_flag(A.err);
 }
 
 template <int NT8, int NW, int CG, bool PRE = true>
-static cudaError_t bjm_launch(const BjArgs &a, const float *X, const float *r, float *z, int32_t *err, cudaStream_t s) {
+static cudaError_t bjm_launch(const BjArgs &a, const float *X, const float *r, float *z, cudaStream_t s) {
   typedef BjmLayout<NT8, NW, PRE> L;
   const void *fn = (const void *)k_bj_mma<NT8, NW, CG, PRE>;
   // two stages unless one leaves room for a second CTA on the SM (or two do not fit)
@@ -392,24 +402,24 @@ static cudaError_t bjm_launch(const BjArgs &a, const float *X, const float *r, f
   at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_bj_mma<NT8, NW, CG, PRE>, a, X, r, z, stages, cs, err);
+  return cudaLaunchKernelEx(&cfg, k_bj_mma<NT8, NW, CG, PRE>, a, X, r, z, stages, cs);
 }
 
 template <int NT8>
-static cudaError_t bjm_by_size(const BjArgs &a, const float *X, const float *r, float *z, int32_t *err, cudaStream_t s) {
-  if (a.n <= 128) return bjm_launch<NT8, 4, 1>(a, X, r, z, err, s);
-  if (a.n <= 256) return bjm_launch<NT8, 4, 2>(a, X, r, z, err, s);
-  if (a.n <= 384) return bjm_launch<NT8, 8, 2>(a, X, r, z, err, s);
-  if (a.n <= 512) return bjm_launch<NT8, 16, 1>(a, X, r, z, err, s);
+static cudaError_t bjm_by_size(const BjArgs &a, const float *X, const float *r, float *z, cudaStream_t s) {
+  if (a.n <= 128) return bjm_launch<NT8, 4, 1>(a, X, r, z, s);
+  if (a.n <= 256) return bjm_launch<NT8, 4, 2>(a, X, r, z, s);
+  if (a.n <= 384) return bjm_launch<NT8, 8, 2>(a, X, r, z, s);
+  if (a.n <= 512) return bjm_launch<NT8, 16, 1>(a, X, r, z, s);
   // up to 8 right-hand sides two CTAs of 8 warps share an SM
-  if (NT8 == 1 && a.n <= 768) return bjm_launch<1, 8, 3>(a, X, r, z, err, s);
-  if (a.n <= 768) return bjm_launch<NT8, 16, 2>(a, X, r, z, err, s);
+  if (NT8 == 1 && a.n <= 768) return bjm_launch<1, 8, 3>(a, X, r, z, s);
+  if (a.n <= 768) return bjm_launch<NT8, 16, 2>(a, X, r, z, s);
   // 16 right-hand sides of r take twice the room in split form: beyond n = 768 they leave
   // none for a second stage (64 blocks of 1000: 110 -> 82 us as FP32 values) or for the first
   // one (64 of 1331: 234 us by 8 right-hand sides per CTA, 162 us so); up to 768 the split at
   // each use costs 5 %
   constexpr bool PRE = NT8 == 1;
-  if (a.n <= 1024) return bjm_launch<NT8, 16, 2, PRE>(a, X, r, z, err, s);
-  if (a.n <= 1536) return bjm_launch<NT8, 16, 3, PRE>(a, X, r, z, err, s);
+  if (a.n <= 1024) return bjm_launch<NT8, 16, 2, PRE>(a, X, r, z, s);
+  if (a.n <= 1536) return bjm_launch<NT8, 16, 3, PRE>(a, X, r, z, s);
   return cudaErrorInvalidValue;
 }

@@ -3,25 +3,25 @@
 #if defined(BJP_F64)
 #include "bj_pass.cuh"
 
-cudaError_t bj_pass_f64(const BjArgs &a, const double *X, const double *r, double *z, int32_t *err, cudaStream_t s) {
+cudaError_t bj_pass_f64(const BjArgs &a, const double *X, const double *r, double *z, cudaStream_t s) {
   if (a.n_group <= 0 || a.n_rhs <= 0) return cudaSuccess;
-  if (a.n_rhs == 1) return bjp_by_size<double, 1>(a, X, r, z, err, s);
+  if (a.n_rhs == 1) return bjp_by_size<double, 1>(a, X, r, z, s);
   // eight right-hand sides per pass where they fit beside one stage of X
-  if (a.n_rhs <= 4 || BjpLayout<double, 8>::bytes(a.n, 1) > 225 * 1024) return bjp_by_size<double, 4>(a, X, r, z, err, s);
-  return bjp_by_size<double, 8>(a, X, r, z, err, s);
+  if (a.n_rhs <= 4 || BjpLayout<double, 8>::bytes(a.n, 1) > 225 * 1024) return bjp_by_size<double, 4>(a, X, r, z, s);
+  return bjp_by_size<double, 8>(a, X, r, z, s);
 }
 #else
 #include "bj_mma.cuh"
 
-cudaError_t bj_pass_f32(const BjArgs &a, const float *X, const float *r, float *z, int32_t *err, cudaStream_t s) {
+cudaError_t bj_pass_f32(const BjArgs &a, const float *X, const float *r, float *z, cudaStream_t s) {
   if (a.n_group <= 0 || a.n_rhs <= 0) return cudaSuccess;
-  if (a.n_rhs == 1) return bjp_by_size<float, 1>(a, X, r, z, err, s);
+  if (a.n_rhs == 1) return bjp_by_size<float, 1>(a, X, r, z, s);
   // blocks up to n = 64 keep FP32 FMAs for any count: their sums are short, and the split of
   // the matrix instructions would be the larger error (against 64 bits, n = 8, 27, 64: 1.2e-7,
   // 1.3e-7, 1.46e-7 against 0.6e-7, 0.97e-7, 1.38e-7 of a chain of FMAs; n = 125: 1.5e-7 against
   // 1.9e-7), although they would be faster on many elements (8,192 of 64, 16 rhs: 90 us, 243 here)
-  if (a.n_rhs <= 4 || a.n <= 64) return bjp_by_size<float, 4>(a, X, r, z, err, s);
-  if (a.n_rhs <= 8) return bjm_by_size<1>(a, X, r, z, err, s);
-  return bjm_by_size<2>(a, X, r, z, err, s);
+  if (a.n_rhs <= 4 || a.n <= 64) return bjp_by_size<float, 4>(a, X, r, z, s);
+  if (a.n_rhs <= 8) return bjm_by_size<1>(a, X, r, z, s);
+  return bjm_by_size<2>(a, X, r, z, s);
 }
 #endif

@@ -19,7 +19,7 @@
 // Bound: FP32 HBM (the factor once: 545 MB for 512 blocks of 729, 80 us; 145 us
 // at 1 and 215 us at 4 right-hand sides, issue-limited), FP64 its pipe (two
 // lanes per clock and SM: 1.73 ms at 4 right-hand sides, 2.42 ms measured).
-// Waits on the copies are bounded: on expiry the CTA sets *err and ends.
+// Waits on the copies are bounded (bj_pass.h).
 #pragma once
 #include <algorithm>
 #include <cmath>
@@ -89,9 +89,8 @@ struct BjpLayout {
 };
 
 __device__ __forceinline__ uint32_t bjp_saddr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ bool bjp_wait(uint32_t bar, uint32_t parity) {
-  // bounded: about a second of polling at most
-  for (int it = 0; it < (1 << 22); ++it) {
+__device__ __forceinline__ bool bjp_wait(uint32_t bar, uint32_t parity, int polls) {
+  for (int it = 0; it < polls; ++it) {
     uint32_t done;
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
@@ -193,7 +192,7 @@ __host__ __device__ constexpr int bjp_per_sm(size_t size, int nth) { return size
 
 template <typename T, int RT, int NTH, int C>
 __global__ void __launch_bounds__(NTH, bjp_per_sm(sizeof(T), NTH))
-    k_bj_pass(BjArgs A, const T *X, const T *in, T *out, int stages, int cs, int32_t *err) {
+    k_bj_pass(BjArgs A, const T *X, const T *in, T *out, int stages, int cs) {
   typedef BjpLayout<T, RT> L;
   constexpr int VR = L::VR, G = L::G, NW = NTH / 32;
   constexpr int MR = BJP_BR / NW;                          // rows of a block per warp
@@ -258,7 +257,7 @@ __global__ void __launch_bounds__(NTH, bjp_per_sm(sizeof(T), NTH))
     for (int q = 0; q < RT; ++q) z[c][q] = (T)0;
   for (int it = 0; it < mine; ++it) {
     const int b = rank + it * cs, i0 = b * BJP_BR, st = stages == 2 ? (it & 1) : 0;
-    if (!bjp_wait(bjp_saddr(&bar[st]), (stages == 2 ? it >> 1 : it) & 1)) s_bad = 1;  // gives up after the barrier below
+    if (!bjp_wait(bjp_saddr(&bar[st]), (stages == 2 ? it >> 1 : it) & 1, A.polls)) s_bad = 1;  // gives up after the barrier below
     const int64_t s0 = xb + bjp_tri(i0);
     const T *Xb = Xs + (size_t)st * stage + (s0 & (AL - 1));  // entry (i0, 0)
     const int dn = min(BJP_BR, n - i0);
@@ -332,8 +331,13 @@ __global__ void __launch_bounds__(NTH, bjp_per_sm(sizeof(T), NTH))
       }
     __syncthreads();
     if (bad) {
-      // wait (bounded) for the other stage's copy before the CTA ends
-      if (stages == 2 && it + 1 < mine) bjp_wait(bjp_saddr(&bar[st ^ 1]), ((it + 1) >> 1) & 1);
+      // the copies in flight land (bounded) before their memory is used again or the CTA ends
+      bjp_wait(bjp_saddr(&bar[st]), (stages == 2 ? it >> 1 : it) & 1, BJ_POLLS);
+      if (stages == 2 && it + 1 < mine) bjp_wait(bjp_saddr(&bar[st ^ 1]), ((it + 1) >> 1) & 1, BJ_POLLS);
+#pragma unroll
+      for (int c = 0; c < C; ++c)
+#pragma unroll
+        for (int q = 0; q < RT; ++q) z[c][q] = (T)__int_as_float(0x7fffffff);
       break;
     }
     if (tid == 0 && it + stages < mine) {
@@ -377,11 +381,11 @@ __global__ void __launch_bounds__(NTH, bjp_per_sm(sizeof(T), NTH))
     }
     asm volatile("barrier.cluster.arrive.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
   }
-  if (tid == 0 && s_bad) atomicExch(err, 1);
+  if (tid == 0 && s_bad) bj_flag(A.err);
 }
 
 template <typename T, int RT, int NTH, int C>
-static cudaError_t bjp_launch(const BjArgs &a, const T *X, const T *r, T *z, int32_t *err, cudaStream_t s) {
+static cudaError_t bjp_launch(const BjArgs &a, const T *X, const T *r, T *z, cudaStream_t s) {
   const void *fn = (const void *)k_bj_pass<T, RT, NTH, C>;
   const int stages = BjpLayout<T, RT>::bytes(a.n, 2) <= 74 * 1024 ? 2 : 1;
   const size_t smem = BjpLayout<T, RT>::bytes(a.n, stages);
@@ -402,26 +406,26 @@ static cudaError_t bjp_launch(const BjArgs &a, const T *X, const T *r, T *z, int
   at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_bj_pass<T, RT, NTH, C>, a, X, r, z, stages, cs, err);
+  return cudaLaunchKernelEx(&cfg, k_bj_pass<T, RT, NTH, C>, a, X, r, z, stages, cs);
 }
 
 template <typename T, int RT>
-static cudaError_t bjp_by_size(const BjArgs &a, const T *X, const T *r, T *z, int32_t *err, cudaStream_t s) {
-  if (a.n <= 64) return bjp_launch<T, RT, 64, 1>(a, X, r, z, err, s);
-  if (a.n <= 128) return bjp_launch<T, RT, 64, 2>(a, X, r, z, err, s);
+static cudaError_t bjp_by_size(const BjArgs &a, const T *X, const T *r, T *z, cudaStream_t s) {
+  if (a.n <= 64) return bjp_launch<T, RT, 64, 1>(a, X, r, z, s);
+  if (a.n <= 128) return bjp_launch<T, RT, 64, 2>(a, X, r, z, s);
   if constexpr (sizeof(T) == 8) {
     // FP64: one CTA per SM from n = 512 on (the X stage), so eight warps to keep its pipe fed
-    if (a.n <= 256) return bjp_launch<T, RT, 128, 2>(a, X, r, z, err, s);
-    if (a.n <= 512) return bjp_launch<T, RT, 256, 2>(a, X, r, z, err, s);
-    if (a.n <= 768) return bjp_launch<T, RT, 256, 3>(a, X, r, z, err, s);
-    if (a.n <= 1024) return bjp_launch<T, RT, 256, 4>(a, X, r, z, err, s);
+    if (a.n <= 256) return bjp_launch<T, RT, 128, 2>(a, X, r, z, s);
+    if (a.n <= 512) return bjp_launch<T, RT, 256, 2>(a, X, r, z, s);
+    if (a.n <= 768) return bjp_launch<T, RT, 256, 3>(a, X, r, z, s);
+    if (a.n <= 1024) return bjp_launch<T, RT, 256, 4>(a, X, r, z, s);
   } else {
-    if (a.n <= 256) return bjp_launch<T, RT, 64, 4>(a, X, r, z, err, s);
-    if (a.n <= 384) return bjp_launch<T, RT, 128, 3>(a, X, r, z, err, s);
-    if (a.n <= 512) return bjp_launch<T, RT, 128, 4>(a, X, r, z, err, s);
-    if (a.n <= 768) return bjp_launch<T, RT, 128, 6>(a, X, r, z, err, s);
-    if (a.n <= 1024) return bjp_launch<T, RT, 128, 8>(a, X, r, z, err, s);
+    if (a.n <= 256) return bjp_launch<T, RT, 64, 4>(a, X, r, z, s);
+    if (a.n <= 384) return bjp_launch<T, RT, 128, 3>(a, X, r, z, s);
+    if (a.n <= 512) return bjp_launch<T, RT, 128, 4>(a, X, r, z, s);
+    if (a.n <= 768) return bjp_launch<T, RT, 128, 6>(a, X, r, z, s);
+    if (a.n <= 1024) return bjp_launch<T, RT, 128, 8>(a, X, r, z, s);
   }
-  if (a.n <= 1536) return bjp_launch<T, RT, 256, 6>(a, X, r, z, err, s);
+  if (a.n <= 1536) return bjp_launch<T, RT, 256, 6>(a, X, r, z, s);
   return cudaErrorInvalidValue;
 }

@@ -12,10 +12,23 @@ struct BjArgs {
   int64_t ndof;            // stride between right-hand sides of a vector
   const int64_t *dof_off;  // per element
   const int64_t *blk_off;  // per element: offset of its packed block
+  int32_t *err;            // host-mapped, set when a bounded wait expired
+  int32_t polls;           // polls after which a wait gives up
 };
+
+// Waits of the block products are bounded: BJ_POLLS polls (about a second; tests
+// lower the limit of the first wait, never that of the one before the CTA ends).
+// An expired wait sets *err, lets what the CTA still has in flight land (bounded
+// too) and leaves NaN in the CTA's part of z.
+constexpr int BJ_POLLS = 1 << 22;
+#if defined(__CUDACC__)
+__device__ __forceinline__ void bj_flag(int32_t *err) {
+  *(volatile int32_t *)err = 1;
+  __threadfence_system();
+}
+#endif
 
 // z = X^T (X r) for the group's elements and all right-hand sides (bj_pass.cuh).
 // X is read in whole 16-byte words: its allocation extends to the next one.
-// err: int32 on the device, set when a bounded wait expired.
-cudaError_t bj_pass_f32(const BjArgs &a, const float *X, const float *r, float *z, int32_t *err, cudaStream_t s);
-cudaError_t bj_pass_f64(const BjArgs &a, const double *X, const double *r, double *z, int32_t *err, cudaStream_t s);
+cudaError_t bj_pass_f32(const BjArgs &a, const float *X, const float *r, float *z, cudaStream_t s);
+cudaError_t bj_pass_f64(const BjArgs &a, const double *X, const double *r, double *z, cudaStream_t s);

@@ -30,8 +30,9 @@
 // issues the 12 MMAs of a chunk (4 K-steps of 8 x 3 products, M = 128, N = 64)
 // and commits them to the stage's mbarrier; the accumulator (128 lanes x 64
 // columns of TMEM) is read back by all four warps (32 lanes each) and stored
-// coalesced along the rows.  Every wait on an mbarrier is bounded: on expiry the
-// CTA sets *err, stops issuing and still frees its TMEM.
+// coalesced along the rows.  Every wait on an mbarrier is bounded (bj_pass.h): on
+// expiry the CTA stops issuing, waits for the MMAs in flight, sets *err, stores NaN
+// and still frees its TMEM.
 #pragma once
 
 constexpr int BJT = 128;                 // tile edge (rows per CTA, MMA M)
@@ -66,7 +67,8 @@ struct BjTcArgs {
   int64_t ndof;
   const int64_t *dof_off;   // per element
   const int64_t *tile_off;  // per element: offset (floats) of its tile set
-  int32_t *err;             // set when a bounded wait expired
+  int32_t *err;             // host-mapped, set when a bounded wait expired
+  int32_t polls;            // polls after which a wait gives up
 };
 
 __device__ __forceinline__ uint32_t bjt_smem(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -109,9 +111,8 @@ __device__ __forceinline__ void bjt_st16(uint32_t addr, const float (&v)[16]) {
       : "memory");
 }
 
-__device__ __forceinline__ bool bjt_wait(uint32_t bar, uint32_t parity) {
-  // bounded: about a second of polling at most
-  for (int it = 0; it < (1 << 22); ++it) {
+__device__ __forceinline__ bool bjt_wait(uint32_t bar, uint32_t parity, int polls) {
+  for (int it = 0; it < polls; ++it) {
     uint32_t done;
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
@@ -233,7 +234,7 @@ __global__ void __launch_bounds__(BJT_THREADS, BJT_MINB) k_bj_tc(BjTcArgs A, con
   for (int kc = kc0; kc < kc1; ++kc) {
     const int it = kc - kc0, st = it % BJT_STAGES;
     // the MMAs that last read this stage (iteration it - BJT_STAGES) are done
-    if (it >= BJT_STAGES && tid == 0 && !bjt_wait(bjt_smem(&bar[st]), ((it - BJT_STAGES) / BJT_STAGES) & 1))
+    if (it >= BJT_STAGES && tid == 0 && !bjt_wait(bjt_smem(&bar[st]), ((it - BJT_STAGES) / BJT_STAGES) & 1, A.polls))
       s_bad = 1;
     __syncthreads();
     if (s_bad) break;
@@ -271,14 +272,23 @@ __global__ void __launch_bounds__(BJT_THREADS, BJT_MINB) k_bj_tc(BjTcArgs A, con
     }
     last = it;
   }
-  // the last commit covers every MMA issued before it
-  if (tid == 0 && !s_bad && last >= 0 &&
-      !bjt_wait(bjt_smem(&bar[last % BJT_STAGES]), (last / BJT_STAGES) & 1))
-    s_bad = 1;
+  // the last commit covers every MMA issued before it; after an expired wait the MMAs
+  // in flight end (bounded) before the tensor memory is freed
+  if (tid == 0 && last >= 0) {
+    const uint32_t mb = bjt_smem(&bar[last % BJT_STAGES]), par = (last / BJT_STAGES) & 1;
+    if (s_bad || !bjt_wait(mb, par, A.polls)) {
+      s_bad = 1;
+      bjt_wait(mb, par, BJ_POLLS);
+    }
+  }
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  if (!s_bad) {
+  {
     const int row = BJT * bi + 32 * warp + lane;
+    // NaN after an expired wait, chosen per value: stored on a path of its own, the kernel
+    // came out with fewer loads in flight (337 -> 379 us)
+    const bool bad = s_bad;
+    if (bad && tid == 0) bj_flag(A.err);
 #pragma unroll
     for (int c0 = 0; c0 < BJT_N; c0 += 16) {
       if (c0 >= nb) break;
@@ -295,11 +305,9 @@ __global__ void __launch_bounds__(BJT_THREADS, BJT_MINB) k_bj_tc(BjTcArgs A, con
         float *dst = out + (int64_t)(r0 + c0) * A.ndof + vb + row;
 #pragma unroll
         for (int j = 0; j < 16; ++j, dst += A.ndof)
-          if (r0 + c0 + j < A.n_rhs) *dst = __uint_as_float(v[j]);
+          if (r0 + c0 + j < A.n_rhs) *dst = __uint_as_float(bad ? 0x7fffffffu : v[j]);
       }
     }
-  } else if (tid == 0) {
-    atomicExch(A.err, 1);
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();

@@ -22,6 +22,7 @@
 
 #include "hpse.h"
 #include "host_math.h"
+#include "bj_pass.h"
 #include "registry.h"
 
 using namespace hpse;
@@ -152,6 +153,34 @@ static cudaError_t upload_reuse(DevBuf &b, const std::vector<T> &v) {
   return cudaMemcpy(b.p, v.data(), bytes, cudaMemcpyHostToDevice);
 }
 
+// an int32 in pinned host memory that kernels write
+struct MappedFlag {
+  int32_t *h = nullptr, *d = nullptr;
+  MappedFlag() = default;
+  MappedFlag(const MappedFlag &) = delete;
+  MappedFlag &operator=(const MappedFlag &) = delete;
+  ~MappedFlag() {
+    if (h) cudaFreeHost(h);
+  }
+  cudaError_t alloc() {
+    if (h) return cudaSuccess;
+    void *p = nullptr, *q = nullptr;
+    cudaError_t e = cudaHostAlloc(&p, sizeof(int32_t), cudaHostAllocMapped);
+    if (e != cudaSuccess) return e;
+    e = cudaHostGetDevicePointer(&q, p, 0);
+    if (e != cudaSuccess) {
+      cudaFreeHost(p);
+      return e;
+    }
+    h = (int32_t *)p;
+    d = (int32_t *)q;
+    set(0);
+    return cudaSuccess;
+  }
+  void set(int32_t v) { *(volatile int32_t *)h = v; }
+  bool get() const { return h && *(volatile const int32_t *)h != 0; }
+};
+
 template <typename T>
 static cudaError_t upload(DevBuf &b, const std::vector<T> &v) {
   cudaError_t e = b.alloc(v.size() * sizeof(T));
@@ -268,7 +297,10 @@ struct hpse_mesh {
   int bj_var[HPSE_MAX_W + 1][2] = {};  // tile variant of the products per degree and precision (autotuned)
   float bj_ms[HPSE_MAX_W + 1][2][9] = {};  // [BJ_NVAR]  // measured time per variant (ms; 0: not a candidate)
   DevBuf d_bjt, d_bjt_off;    // tensor-core form: FP32 tiles of X and X^T per element, their offsets
-  DevBuf d_bjt_err;           // int32: set by a tensor-core product whose bounded wait expired
+  // set (by the device, in host memory) when a bounded wait of the block products
+  // expired; cleared by the next set-up of the block preconditioner
+  MappedFlag bj_err;
+  int32_t bj_polls = BJ_POLLS;  // polls after which such a wait gives up
   int threads[2][2][HPSE_MAX_W + 1];  // [kind][prec][W]
   // one stream per degree group: per-degree launches of one operator or
   // preconditioner application run concurrently (fork/join through events,
@@ -1181,13 +1213,22 @@ static BjArgs bj_args(const hpse_mesh *m, const Group &g, int n_rhs) {
   a.ndof = m->ndof;
   a.dof_off = m->d_dof_off.as<int64_t>();
   a.blk_off = m->d_bj_off.as<int64_t>();
+  a.err = m->bj_err.d;
+  a.polls = m->bj_polls;
   return a;
+}
+
+// a wait of the block products expired since the preconditioner was set up: z held NaN
+static bool bj_expired(const hpse_mesh *m) { return m->precond_kind == HPSE_PRECOND_BLOCK && m->bj_err.get(); }
+static hpse_status bj_expired_status() {
+  snprintf(g_last_err, sizeof(g_last_err), "a bounded wait of the element-block products expired");
+  return HPSE_ERR_CUDA;
 }
 
 // z = X^T (X r) for a group on the tensor cores (FP32, variant BJ_TC)
 static hpse_status bj_tc_pair(hpse_mesh *m, const Group &g, int n_rhs, const float *r, float *t, float *z,
                               cudaStream_t s) {
-  if (!m->d_bjt.p || !m->d_bjt_err.p) return HPSE_ERR_INVALID_ARG;
+  if (!m->d_bjt.p) return HPSE_ERR_INVALID_ARG;
   BjTcArgs a;
   a.elems = g.elems.as<int32_t>();
   a.n_group = g.n;
@@ -1196,7 +1237,8 @@ static hpse_status bj_tc_pair(hpse_mesh *m, const Group &g, int n_rhs, const flo
   a.ndof = m->ndof;
   a.dof_off = m->d_dof_off.as<int64_t>();
   a.tile_off = m->d_bjt_off.as<int64_t>();
-  a.err = m->d_bjt_err.as<int32_t>();
+  a.err = m->bj_err.d;
+  a.polls = m->bj_polls;
   const dim3 grid(g.n * ((a.n + BJT - 1) / BJT), (n_rhs + BJT_N - 1) / BJT_N);
   k_bj_tc<false><<<grid, BJT_THREADS, BJT_SMEM, s>>>(a, m->d_bjt.as<float>(), r, t);
   k_bj_tc<true><<<grid, BJT_THREADS, BJT_SMEM, s>>>(a, m->d_bjt.as<float>(), t, z);
@@ -1211,8 +1253,8 @@ static hpse_status bj_products(hpse_mesh *m, const Group &g, const BjArgs &a, co
     if (v == BJ_TC) return bj_tc_pair(m, g, a.n_rhs, r, t, z, s);
   }
   if (bj_is_pass(v, sizeof(T) == 4)) {
-    if constexpr (sizeof(T) == 4) CK(bj_pass_f32(a, X, r, z, m->d_bjt_err.as<int32_t>(), s));
-    else CK(bj_pass_f64(a, X, r, z, m->d_bjt_err.as<int32_t>(), s));
+    if constexpr (sizeof(T) == 4) CK(bj_pass_f32(a, X, r, z, s));
+    else CK(bj_pass_f64(a, X, r, z, s));
     return HPSE_OK;
   }
   CK(bj_apply_group<T>(a, X, r, t, z, s, v));
@@ -2912,6 +2954,7 @@ extern "C" hpse_status hpse_apply_preconditioner(hpse_mesh *m, int32_t prec, con
   if (!m || (prec != HPSE_FP64 && prec != HPSE_FP32)) return HPSE_ERR_INVALID_ARG;
   if (m->ndof == 0) return HPSE_OK;
   if (!r || !z || r == z) return HPSE_ERR_INVALID_ARG;
+  if (bj_expired(m)) return bj_expired_status();
   CK(cudaSetDevice(m->device));
   cudaStream_t s = (cudaStream_t)stream;
   if (prec == HPSE_FP64) {
@@ -2941,6 +2984,8 @@ extern "C" hpse_status hpse_setup_block_preconditioner(hpse_mesh *m) {
   drop_graphs(m);
   m->bj_ready = false;
   m->precond_kind = HPSE_PRECOND_SEPARABLE;
+  CK(m->bj_err.alloc());
+  m->bj_err.set(0);
   const int E = m->n_elem;
   std::vector<int64_t> off(E + 1, 0);
   for (int e = 0; e < E; ++e) {
@@ -3030,8 +3075,6 @@ extern "C" hpse_status hpse_setup_block_preconditioner(hpse_mesh *m) {
   int32_t h_fail = 0;
   CK(cudaMemcpy(&h_fail, fail.p, sizeof(int32_t), cudaMemcpyDeviceToHost));
   if (h_fail) return HPSE_ERR_BREAKDOWN;
-  if (!m->d_bjt_err.p) CK(m->d_bjt_err.alloc(sizeof(int32_t)));
-  CK(cudaMemset(m->d_bjt_err.p, 0, sizeof(int32_t)));
   // tensor-core form (a candidate from 32 right-hand sides on): FP32 tiles of
   // X and X^T per element
   m->d_bjt = DevBuf();
@@ -3076,6 +3119,7 @@ extern "C" hpse_status hpse_setup_block_preconditioner(hpse_mesh *m) {
         const int nc2 = bj_candidates(m->n_rhs, pi == 1, cand);
         float best = 1e30f;
         for (int k = 0; k < BJ_NVAR; ++k) m->bj_ms[g.W][pi][k] = 0.0f;
+        m->bj_var[g.W][pi] = 0;  // a tile of both precisions and any count, if no candidate is left
         for (int ci = 0; ci < nc2; ++ci) {
           const int v = cand[ci];
           if (v == BJ_TC && !m->d_bjt.p) continue;
@@ -3094,11 +3138,10 @@ extern "C" hpse_status hpse_setup_block_preconditioner(hpse_mesh *m) {
           CK(cudaEventSynchronize(e1));
           CK(cudaEventElapsedTime(&ms, e0, e1));
           ms /= 3.0f;
-          if (v == BJ_TC || bj_is_pass(v, pi == 1)) {
+          if (m->bj_err.get()) {
             // a product whose bounded wait expired is not a candidate
-            int32_t h_err = 0;
-            CK(cudaMemcpy(&h_err, m->d_bjt_err.p, sizeof(int32_t), cudaMemcpyDeviceToHost));
-            if (h_err) continue;
+            m->bj_err.set(0);
+            continue;
           }
           m->bj_ms[g.W][pi][v] = ms;
           if (ms < best) {
@@ -3142,6 +3185,7 @@ extern "C" hpse_status hpse_setup_block_preconditioner(hpse_mesh *m) {
       double h[2] = {0.0, 0.0};
       CK(cudaMemcpyAsync(h, acc.p, 2 * sizeof(double), cudaMemcpyDeviceToHost, s));
       CK(cudaStreamSynchronize(s));
+      if (m->bj_err.get()) return bj_expired_status();
       const double rel = h[1] > 0.0 ? std::sqrt(h[0] / h[1]) : 0.0;
       m->bj_poor32[g.W] = !(rel <= 1e-2);
       any_poor = any_poor || m->bj_poor32[g.W];
@@ -3180,6 +3224,15 @@ extern "C" hpse_status hpse_set_block_tile(hpse_mesh *m, int32_t W, int32_t prec
   CK(cudaDeviceSynchronize());
   drop_graphs(m);
   m->bj_var[W][prec == HPSE_FP64 ? 0 : 1] = variant;
+  return HPSE_OK;
+}
+
+extern "C" hpse_status hpse_set_block_wait(hpse_mesh *m, int32_t polls) {
+  if (!m || polls < 0 || polls > BJ_POLLS) return HPSE_ERR_INVALID_ARG;
+  CK(cudaSetDevice(m->device));
+  CK(cudaDeviceSynchronize());
+  drop_graphs(m);
+  m->bj_polls = polls;
   return HPSE_OK;
 }
 
@@ -3375,7 +3428,7 @@ static hpse_status run_pcg(hpse_mesh *m, T *x, T *r, T *z, T *pa, T *pb, T *q, d
     CK(cudaMemcpyAsync(w.h_flags, w.flags.p, (size_t)(3 * npr + 1) * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
     const int n_active = w.h_flags[3 * npr];
-    if (n_active == 0) break;
+    if (n_active == 0 || bj_expired(m)) break;
     if (done >= max_iter) {
       *status = HPSE_ERR_NO_CONVERGENCE;
       break;
@@ -3549,6 +3602,7 @@ static hpse_status solve_reliable(hpse_mesh *m, const hpse_solve_opts *o, double
     CK(cudaMemcpyAsync(w.h_flags, w.flags.p, (size_t)(3 * npr + 1) * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
     CK(cudaMemcpyAsync(w.h_sc, w.sc.p, (size_t)12 * npr * sizeof(double), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
+    if (bj_expired(m)) break;  // hpse_pcg_solve reports it
     const int n_active = w.h_flags[3 * npr];
     bool refresh = n_active == 0;
     for (int i = 0; i < npr && !refresh; ++i)
@@ -3641,14 +3695,14 @@ static hpse_status solve_reliable(hpse_mesh *m, const hpse_solve_opts *o, double
   return HPSE_OK;
 }
 
-extern "C" hpse_status hpse_pcg_solve(hpse_mesh *m, const hpse_solve_opts *o, double *x, hpse_solve_report *rep,
-                                      void *stream) {
+static hpse_status pcg_solve(hpse_mesh *m, const hpse_solve_opts *o, double *x, hpse_solve_report *rep, void *stream) {
   if (!m || !o || !rep) return HPSE_ERR_INVALID_ARG;
   memset(rep, 0, sizeof(*rep));
   if (!m->has_data) return HPSE_ERR_NO_DATA;
   if (!(o->tol > 0.0) || o->max_iter < 1 || (o->prec != HPSE_FP64 && o->prec != HPSE_FP32)) return HPSE_ERR_INVALID_ARG;
   if (m->ndof == 0) return HPSE_OK;
   if (!x) return HPSE_ERR_INVALID_ARG;
+  if (bj_expired(m)) return bj_expired_status();
   CK(cudaSetDevice(m->device));
   hpse_status st = ensure_work(m);
   if (st != HPSE_OK) return st;
@@ -3759,6 +3813,7 @@ extern "C" hpse_status hpse_pcg_solve(hpse_mesh *m, const hpse_solve_opts *o, do
       total_it += it;
       applies += it;
       ++sweeps;
+      if (bj_expired(m)) break;
       if (ist == HPSE_ERR_BREAKDOWN) {
         status = ist;
         break;
@@ -3785,6 +3840,17 @@ extern "C" hpse_status hpse_pcg_solve(hpse_mesh *m, const hpse_solve_opts *o, do
   rep->applies = applies;
   rep->status = status;
   return (hpse_status)status;
+}
+
+extern "C" hpse_status hpse_pcg_solve(hpse_mesh *m, const hpse_solve_opts *o, double *x, hpse_solve_report *rep,
+                                      void *stream) {
+  const hpse_status st = pcg_solve(m, o, x, rep, stream);
+  // every way out has waited for the solver's stream: an expired wait of this solve is known
+  if (m && o && rep && bj_expired(m)) {
+    rep->status = HPSE_ERR_CUDA;
+    return bj_expired_status();
+  }
+  return st;
 }
 
 extern "C" hpse_status hpse_h1_error(hpse_mesh *m, const double *u, const double *ref, const double *vq,
