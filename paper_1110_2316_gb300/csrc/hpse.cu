@@ -254,12 +254,13 @@ struct hpse_mesh {
   std::vector<Group> groups;
   // device mesh arrays
   // d_prob: problem of each vector item (n_elem + n_corner entries)
-  DevBuf d_dof_off, d_nbr, d_geo64, d_geo32, d_sqj64, d_sqj32, d_prob, d_coef_off, d_prob_ptr, d_prob_elems, d_elem_W;
+  DevBuf d_dof_off, d_nbr, d_geo64, d_geo32, d_prob, d_coef_off, d_prob_ptr, d_prob_elems, d_elem_W;
   DevBuf d_coef64, d_coef32;  // [nquad][4] (m, d_x, d_y, d_z) per point (COEF_SCALAR);
                               // [nquad][12] (w J, C_11 .. C_0, 0) (HPSE_COEF_GENERAL)
   DevBuf d_b;                 // FP64 right-hand side
   DevBuf d_f;                 // FP64 source at the volume points [n_rhs][nquad]
   DevBuf d_aux;               // FP64 [5][nquad]: w J, a, a_x, a_y, a_z at the volume points
+  DevBuf d_sqw64, d_sqw32;    // [nquad] sqrt(w J) of the residual map (box meshes, not the general operator)
   DevBuf d_tabs_ptr;          // device array of the per-degree FP64 table pointers
   DevBuf d_scr_rho;           // scratch of the integration-by-parts transpose
   // conforming correction (box meshes; built on first use): per element corner
@@ -2357,8 +2358,7 @@ extern "C" hpse_status hpse_setup_mesh(const hpse_mesh_desc *d, int device, hpse
     }
   }
   std::vector<double> geo(4 * (size_t)E);
-  std::vector<float> geo32(4 * (size_t)E), sqj32(E);
-  std::vector<double> sqj(E);  // square roots of the Jacobians (residual map)
+  std::vector<float> geo32(4 * (size_t)E);
   for (int e = 0; e < E; ++e) {
     double J = 1.0;
     for (int a = 0; a < 3; ++a) {
@@ -2368,8 +2368,6 @@ extern "C" hpse_status hpse_setup_mesh(const hpse_mesh_desc *d, int device, hpse
     }
     geo[4 * e + 3] = J;
     for (int k = 0; k < 4; ++k) geo32[4 * e + k] = (float)geo[4 * e + k];
-    sqj[e] = std::sqrt(geo[4 * e + 3]);
-    sqj32[e] = (float)sqj[e];
   }
   if (nbhd) {
     hpse_status st = setup_edge(m.get());
@@ -2381,8 +2379,6 @@ extern "C" hpse_status hpse_setup_mesh(const hpse_mesh_desc *d, int device, hpse
   CK(upload(m->d_nbr, m->nbr));
   CK(upload(m->d_geo64, geo));
   CK(upload(m->d_geo32, geo32));
-  CK(upload(m->d_sqj64, sqj));
-  CK(upload(m->d_sqj32, sqj32));
   if (m->has_nr || m->has_mixed || m->curved) {
     std::vector<float> g32(m->fgam.begin(), m->fgam.end());
     CK(upload(m->d_fbc, m->fbc));
@@ -2624,6 +2620,15 @@ __global__ void k_coef_general(int64_t nq, const int32_t *elem_W, const int64_t 
   }
 }
 
+// sqrt(w J) at the volume points, FP64 and its FP32 rounding
+__global__ void k_sqrt_wj(int64_t nq, const double *wj, double *s64, float *s32) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nq; i += (int64_t)gridDim.x * blockDim.x) {
+    const double v = sqrt(wj[i]);
+    s64[i] = v;
+    s32[i] = (float)v;
+  }
+}
+
 // where a data pointer points: 1 device (or managed), 0 host, -1 unknown
 static int pointer_space(const void *p) {
   cudaPointerAttributes at;
@@ -2808,6 +2813,13 @@ extern "C" hpse_status hpse_set_data(hpse_mesh *m, const hpse_data *data, void *
       CK(upload_reuse(m->d_coef32, c32));
     }
     CK(upload(dwja, wja));
+  }
+  if (m->coord == HPSE_COORD_CARTESIAN && !gen && nq > 0) {
+    if (m->d_sqw64.bytes != (size_t)nq * sizeof(double)) CK(m->d_sqw64.alloc((size_t)nq * sizeof(double)));
+    if (m->d_sqw32.bytes != (size_t)nq * sizeof(float)) CK(m->d_sqw32.alloc((size_t)nq * sizeof(float)));
+    k_sqrt_wj<<<1024, 256, 0, s>>>(nq, m->d_aux.as<double>(), m->d_sqw64.as<double>(), m->d_sqw32.as<float>());
+    CK(cudaGetLastError());
+    ++g_launches;
   }
   const size_t nv = (size_t)R * m->ndof;
   if (!m->d_b.p || m->d_b.bytes != nv * sizeof(double)) CK(m->d_b.alloc(nv * sizeof(double)));
@@ -4302,7 +4314,7 @@ template <typename T>
 static hpse_status residual_t(hpse_mesh *m, const T *u, T *z, cudaStream_t s) {
   ApplyArgsT<T> a = apply_args<T>(m, m->groups[0], u, nullptr);
   a.aux = m->d_aux.as<double>();
-  a.sqj = (sizeof(T) == 8) ? (const T *)m->d_sqj64.p : (const T *)m->d_sqj32.p;
+  a.sqw64 = m->d_sqw64.as<double>();
   a.f = m->d_f.as<double>();
   a.zout = z;
   a.skip_faces = 1;
@@ -4326,7 +4338,7 @@ template <typename T>
 static hpse_status transpose_t(hpse_mesh *m, const T *z, T *y, cudaStream_t s) {
   ApplyArgsT<T> a = apply_args<T>(m, m->groups[0], nullptr, y);
   a.aux = m->d_aux.as<double>();
-  a.sqj = (sizeof(T) == 8) ? (const T *)m->d_sqj64.p : (const T *)m->d_sqj32.p;
+  a.sqw = (sizeof(T) == 8) ? (const T *)m->d_sqw64.p : (const T *)m->d_sqw32.p;
   a.zin = z;
   a.skip_faces = 1;
   return launch_apply_all<T>(m, MODE_TRANSPOSE, a, s);

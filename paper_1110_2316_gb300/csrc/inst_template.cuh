@@ -3,7 +3,6 @@
 // HPSE_REGISTER_NAME (and HPSE_DOUBLE for REAL = double), then includes this.
 // HPSE_APPLY_ONLY with HPSE_APPLY_NT, HPSE_LINES_NC: the apply kernels alone in a
 // second launch shape.
-#include <cmath>
 #include <vector>
 
 #include "kernels.cuh"
@@ -171,7 +170,6 @@ cudaError_t upload_fn(const double *pk) {
         t.PF[m][0][i * HPE + j] = (real)(mid ? x(i, j) : 0.5 * (x(i, j) + x(i, P - 1 - j)));
         t.PF[m][1][i * HPE + j] = (real)(mid ? 0.0 : 0.5 * (x(i, j) - x(i, P - 1 - j)));
       }
-  for (int i = 0; i < Q; ++i) t.SQ[i] = (real)std::sqrt(pk[o + i]);
   for (int i = 0; i < Q; ++i) t.WQ[i] = (real)pk[o++];
   for (int i = 0; i < P; ++i) t.MU[i] = (real)pk[o++];
   cudaError_t err = cudaMemcpyToSymbol(c_tab, &t, sizeof(Tables));

@@ -122,7 +122,6 @@ struct Tables {
   real MP[P2];
   real KP[P2];
   real WQ[Q];
-  real SQ[Q];  // square roots of WQ
   real MU[P];
   // pairs of folded entries for the packed FP32 contractions (two matrices
   // applied at once, see fwd_pm2): XE[0][i] = (FE[0][i], FE[0][i]),
@@ -1479,23 +1478,27 @@ __global__ void __launch_bounds__(NT, APPLY_MINB) k_apply(const ApplyArgs A) {
     std::conditional_t<inplace, ColumnRhoT<TS>, ColumnRho<L::RHO_SMEM>> rho;
     if constexpr (inplace) rho.bind(sT, l, ok);
     else rho.bind(srho, ok ? l : Q2);
-    // -sqrt(w J) of the column's points but for its factor along z (residual map and its transpose)
-    real swab = 0;
-    if (MODE == MODE_RESIDUAL || (MODE == MODE_TRANSPOSE && A.zin)) swab = -c_tab.SQ[qa] * c_tab.SQ[qb] * A.sqj[e];
+    // sqrt(w J) of the residual map and its transpose comes per point, rounded once (as a
+    // product of four tabulated square roots: up to 1.4 times the FP32 error, W = 3), and the
+    // residual is put together in 64 bits, which its data come in: one rounding in place of
+    // five makes up for those of the folded contractions (FP32, W = 4: 1.09e-7 -> 1.02e-7,
+    // 0.98e-7 without folding; W = 8: 1.20 -> 1.11, 1.14).  It costs 4 rhs of 512 elements of
+    // W = 8 some FP64 time in FP32: 97 -> 131 us.
     auto emit = [&](int q, real sigma) {  // sigma: L u = -a sigma
       const int64_t o = cbase + (int64_t)q * Q2;
-      real v = (real)A.f[(int64_t)r * A.nquad + o];
-      v += var_coef(COEF) ? (real)A.aux[A.nquad + o] * sigma : sigma;
-      if (ok) A.zout[(int64_t)r * A.nquad + o] = swab * c_tab.SQ[q] * v;
+      double v = hpse::widen(sigma);
+      if (var_coef(COEF)) v *= A.aux[A.nquad + o];
+      v += A.f[(int64_t)r * A.nquad + o];
+      if (ok) A.zout[(int64_t)r * A.nquad + o] = (real)(-A.sqw64[o] * v);
     };
     if (MODE == MODE_TRANSPOSE) {
       if (A.zin) {
 #pragma unroll
         for (int qc = 0; qc < Q; ++qc) {
           const int64_t o = cbase + (int64_t)qc * Q2;
-          real v = A.zin[(int64_t)r * A.nquad + o];
+          real v = -A.sqw[o];
           if (var_coef(COEF)) v *= (real)A.aux[A.nquad + o];
-          rho[qc] = swab * c_tab.SQ[qc] * v;
+          rho[qc] = v * A.zin[(int64_t)r * A.nquad + o];
         }
       } else {
 #pragma unroll

@@ -72,7 +72,8 @@ struct ApplyArgsT {
   // source f, the point values written (MODE_RESIDUAL) or transposed (MODE_TRANSPOSE)
   const double *aux;
   const double *f;
-  const T *sqj;             // [E] square root of the element's Jacobian
+  const double *sqw64;      // [nquad] square root of w J
+  const T *sqw;
   T *zout;
   const T *zin;
   int32_t skip_faces;
