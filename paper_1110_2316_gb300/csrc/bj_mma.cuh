@@ -1,6 +1,6 @@
 // bj_mma.cuh -- the one-pass product z = X^T (X r) (bj_pass.cuh) for 5 to 31
-// FP32 right-hand sides of blocks above n = 64: the same walk over blocks of 16 rows of X, with the
-// products on mma.sync m16n8k8 (TF32).  At 8 and 16 right-hand sides the packed
+// FP32 right-hand sides (variant 2: any count from 32 on) of blocks above n = 256:
+// the same walk over blocks of 16 rows of X, with the products on mma.sync m16n8k8 (TF32).  At 8 and 16 right-hand sides the packed
 // FMAs and their shared loads bound the pass (271 and 480 us for 512 blocks of
 // 729); the matrix instructions cut the issued instructions, so that what is
 // left is the reading of X, its split and the latency of a block (242 and
@@ -407,8 +407,6 @@ static cudaError_t bjm_launch(const BjArgs &a, const float *X, const float *r, f
 
 template <int NT8>
 static cudaError_t bjm_by_size(const BjArgs &a, const float *X, const float *r, float *z, cudaStream_t s) {
-  if (a.n <= 128) return bjm_launch<NT8, 4, 1>(a, X, r, z, s);
-  if (a.n <= 256) return bjm_launch<NT8, 4, 2>(a, X, r, z, s);
   if (a.n <= 384) return bjm_launch<NT8, 8, 2>(a, X, r, z, s);
   if (a.n <= 512) return bjm_launch<NT8, 16, 1>(a, X, r, z, s);
   // up to 8 right-hand sides two CTAs of 8 warps share an SM
