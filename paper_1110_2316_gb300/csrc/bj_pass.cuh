@@ -261,7 +261,18 @@ __global__ void __launch_bounds__(NTH, bjp_per_sm(sizeof(T), NTH))
     const int64_t s0 = xb + bjp_tri(i0);
     const T *Xb = Xs + (size_t)st * stage + (s0 & (AL - 1));  // entry (i0, 0)
     const int dn = min(BJP_BR, n - i0);
-    // t = X r: warp w takes rows i0 + MR w + m, its lanes the columns
+    // t = X r: warp w takes rows i0 + MR w + m, its lanes the columns.  Of a block of one row
+    // block (W = 1) one thread sums a row in turn: over lanes every product of the few terms
+    // is rounded by itself (FP32, n = 8: error 7.2e-8, a chain of FMAs 6.2e-8)
+    if (C == 1 && n <= BJP_BR) {
+      for (int idx = tid; idx < dn * RT; idx += NTH) {
+        const int d = idx / RT, q = idx - d * RT;
+        const T *rq = rs + (size_t)(q / VR) * n32 * VR + q % VR;
+        T s = (T)0;
+        for (int k = 0; k <= d; ++k) s += Xb[bjp_tri(d) + k] * rq[k * VR];
+        ts[idx] = s;
+      }
+    } else
 #pragma unroll
     for (int q0 = 0; q0 < RT; q0 += RP) {
       T acc[MR * RP];

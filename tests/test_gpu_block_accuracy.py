@@ -45,7 +45,7 @@ def _errors(api, m, W, r, variants):
 
 
 # three elements (a cluster of CTAs per element), and enough of them for a CTA per element
-@pytest.mark.parametrize("W,boxes", [(W, (3, 1, 1)) for W in range(2, 11)] + [(4, (10, 8, 5)), (6, (7, 7, 6))])
+@pytest.mark.parametrize("W,boxes", [(W, (3, 1, 1)) for W in range(1, 11)] + [(4, (10, 8, 5)), (6, (7, 7, 6))])
 @pytest.mark.parametrize("n_rhs", [7, 16, 31])
 def test_error_no_larger_than_the_tiles(api, W, boxes, n_rhs):
     m = _mesh(api, W, boxes, n_rhs)
