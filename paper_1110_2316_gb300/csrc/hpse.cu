@@ -1244,6 +1244,7 @@ static hpse_status bj_tc_pair(hpse_mesh *m, const Group &g, int n_rhs, const flo
   k_bj_tc<false><<<grid, BJT_THREADS, BJT_SMEM, s>>>(a, m->d_bjt.as<float>(), r, t);
   k_bj_tc<true><<<grid, BJT_THREADS, BJT_SMEM, s>>>(a, m->d_bjt.as<float>(), t, z);
   CK(cudaGetLastError());
+  g_launches += 2;
   return HPSE_OK;
 }
 
@@ -1256,9 +1257,11 @@ static hpse_status bj_products(hpse_mesh *m, const Group &g, const BjArgs &a, co
   if (bj_is_pass(v, sizeof(T) == 4)) {
     if constexpr (sizeof(T) == 4) CK(bj_pass_f32(a, X, r, z, s));
     else CK(bj_pass_f64(a, X, r, z, s));
+    ++g_launches;
     return HPSE_OK;
   }
   CK(bj_apply_group<T>(a, X, r, t, z, s, v));
+  g_launches += 2;
   return HPSE_OK;
 }
 
@@ -1333,11 +1336,10 @@ static hpse_status launch_bj_all(hpse_mesh *m, int mode, const PrecArgsT<T> &b, 
       if (st != HPSE_OK) return st;
       k_bj_cvt<double, T><<<items, 128, 0, gs>>>(a, m->bj_z64.as<double>(), b.zout);
       CK(cudaGetLastError());
-      g_launches += 4;
+      g_launches += 2;
     } else {
       hpse_status st = bj_products<T>(m, g, a, X, rin, t, b.zout, gs, m->bj_var[g.W][sizeof(T) == 8 ? 0 : 1]);
       if (st != HPSE_OK) return st;
-      g_launches += 2;
     }
     if (mode == MODE_PCG) {
       k_bj_dot<T><<<bj_vec_grid(items), 32 * BJ_VEC_ITEMS, 0, gs>>>(a, b.zout, b.r, b.part_rz);
@@ -3144,7 +3146,6 @@ extern "C" hpse_status hpse_setup_block_preconditioner(hpse_mesh *m) {
                         : bj_products<float>(m, g, ba, m->d_bj32.as<float>(), tin.as<float>(), m->bj_t32.as<float>(),
                                              tout.as<float>(), s, v);
             if (st != HPSE_OK) return st;
-            g_launches += 2;
           }
           CK(cudaEventRecord(e1, s));
           CK(cudaEventSynchronize(e1));
@@ -3187,13 +3188,13 @@ extern "C" hpse_status hpse_setup_block_preconditioner(hpse_mesh *m) {
       hpse_status st = bj_products<double>(m, g, ba, m->d_bj64.as<double>(), v64.as<double>(), m->bj_t64.as<double>(),
                                            z64.as<double>(), s, m->bj_var[g.W][0]);
       if (st != HPSE_OK) return st;
-      st = bj_products<float>(m, g, ba, m->d_bj32.as<float>(), v32.as<float>(),
-                                                m->bj_t32.as<float>(), z32.as<float>(), s, m->bj_var[g.W][1]);
+      st = bj_products<float>(m, g, ba, m->d_bj32.as<float>(), v32.as<float>(), m->bj_t32.as<float>(),
+                              z32.as<float>(), s, m->bj_var[g.W][1]);
       if (st != HPSE_OK) return st;
       CK(cudaMemsetAsync(acc.p, 0, 2 * sizeof(double), s));
       k_bj_cmp<<<g.n * m->n_rhs, 128, 0, s>>>(ba, z32.as<float>(), z64.as<double>(), acc.as<double>());
       CK(cudaGetLastError());
-      g_launches += 5;
+      ++g_launches;
       double h[2] = {0.0, 0.0};
       CK(cudaMemcpyAsync(h, acc.p, 2 * sizeof(double), cudaMemcpyDeviceToHost, s));
       CK(cudaStreamSynchronize(s));
