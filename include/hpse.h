@@ -347,7 +347,8 @@ hpse_status hpse_setup_block_preconditioner(hpse_mesh *m);
  * tensor cores (tcgen05, 128 rows x 64 right-hand sides per CTA, each FP32
  * operand split into two TF32 parts, three MMAs per product, FP32
  * accumulation in tensor memory).  hpse_block_tile returns the chosen
- * variant, its tile (rows x right-hand sides per CTA) and, if ms is not NULL,
+ * variant, its tile (rows x right-hand sides per CTA; a one-pass variant works on all
+ * (W+1)^3 rows of a block) and, if ms is not NULL,
  * the measured milliseconds of each of the 9 variants (0 for those not tried);
  * HPSE_ERR_NO_DATA before the set-up.  hpse_set_block_tile overrides the
  * choice (HPSE_ERR_INVALID_ARG for a variant that does not exist in that

@@ -32,3 +32,6 @@ __device__ __forceinline__ void bj_flag(int32_t *err) {
 // X is read in whole 16-byte words: its allocation extends to the next one.
 cudaError_t bj_pass_f32(const BjArgs &a, const float *X, const float *r, float *z, cudaStream_t s);
 cudaError_t bj_pass_f64(const BjArgs &a, const double *X, const double *r, double *z, cudaStream_t s);
+// right-hand sides that one CTA of the above takes, for blocks of size n
+int bj_pass_rhs_f32(int n, int n_rhs);
+int bj_pass_rhs_f64(int n, int n_rhs);

@@ -3222,8 +3222,11 @@ extern "C" hpse_status hpse_block_tile(const hpse_mesh *m, int32_t W, int32_t pr
   if (!m->bj_ready) return HPSE_ERR_NO_DATA;
   const int pi = prec == HPSE_FP64 ? 0 : 1, v = m->bj_var[W][pi];
   if (variant) *variant = v;
-  if (tile_rows) *tile_rows = BJ_TILE[v][0];
-  if (tile_rhs) *tile_rhs = BJ_TILE[v][1];
+  const bool pass = bj_is_pass(v, prec == HPSE_FP32);
+  const int n = (W + 1) * (W + 1) * (W + 1);
+  if (tile_rows) *tile_rows = pass ? n : BJ_TILE[v][0];
+  if (tile_rhs)
+    *tile_rhs = !pass ? BJ_TILE[v][1] : (prec == HPSE_FP32 ? bj_pass_rhs_f32(n, m->n_rhs) : bj_pass_rhs_f64(n, m->n_rhs));
   if (ms)
     for (int k = 0; k < BJ_NVAR; ++k) ms[k] = m->bj_ms[W][pi][k];
   return HPSE_OK;
