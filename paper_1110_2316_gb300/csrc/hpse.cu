@@ -1361,8 +1361,7 @@ static hpse_status launch_prec_all(hpse_mesh *m, int mode, PrecArgsT<T> base_arg
     a.elems = g.elems.as<int32_t>();
     a.n_group = g.n;
     const KernelSet &ks = g_sets[pi][g.W];
-    const int th = m->threads[1][pi][g.W];
-    CK(ks.precond(mode, &a, g.n * m->n_rhs, th, group_stream(m, gi, s)));
+    CK(ks.precond(mode, &a, g.n * m->n_rhs, m->n_sm, group_stream(m, gi, s)));
     ++g_launches;
   }
   CK(group_join(m, s));

@@ -80,10 +80,10 @@ cudaError_t launch_precond_t(const void *args, int n_items, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-cudaError_t precond_fn(int mode, const void *args, int n_items, int threads, cudaStream_t s) {
+cudaError_t precond_fn(int mode, const void *args, int n_items, int sms, cudaStream_t s) {
   if (n_items <= 0) return cudaSuccess;
-  (void)threads;  // CTA shape fixed at compile time: items of PC_TPI threads
-  const bool few = PC_ITEMS > 1 && n_items < PC_FEW;
+  // CTA shape fixed at compile time (items of PC_TPI threads); fewer CTAs than twice the SMs: one item each
+  const bool few = PC_ITEMS > 1 && n_items < 2 * sms * PC_ITEMS;
   if (mode == MODE_PLAIN)
     return few ? launch_precond_t<MODE_PLAIN, 1>(args, n_items, s) : launch_precond_t<MODE_PLAIN, PC_ITEMS>(args, n_items, s);
   if (mode == MODE_PCG)

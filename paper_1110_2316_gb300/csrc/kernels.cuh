@@ -1820,11 +1820,11 @@ __global__ void __launch_bounds__(NT, APPLY_MINB) k_apply(const ApplyArgs A) {
 // would fill fewer CTAs than twice the SMs take one item per CTA instead: an
 // FP64 item alone is bound by its SM's FP64 pipe (two lanes per clock), so six
 // items on one SM and none on the next cost six times (128 FP64 items of W = 6:
-// 45 -> 19 us, 1,024: 84 -> 53 us; FP32 stays at the launch's latency).
+// 45 -> 19 us, 1,024: 84 -> 53 us; FP32 stays at the launch's latency).  Counted per
+// degree group, as measured; groups that run at the same time are not added up.
 constexpr int PC_TPI = PAD32(P2);
 constexpr int PC_ITEMS_RAW = 384 / PC_TPI;
 constexpr int PC_ITEMS = PC_ITEMS_RAW < 1 ? 1 : (PC_ITEMS_RAW > 8 ? 8 : PC_ITEMS_RAW);
-constexpr int PC_FEW = 304 * PC_ITEMS;
 constexpr int PC_WARPS_PER_ITEM = PC_TPI / 32;
 // per item: two P^3 blocks; then the reduction buffer; then per item the x3
 // eigenbasis and eigenvalues of the C* form (edge neighbourhood)

@@ -146,8 +146,8 @@ struct KernelSet {
   cudaError_t (*apply)(int coef, int mode, const void *args, int n_items, int threads, cudaStream_t s);
   size_t (*apply_smem)(int coef);
   int (*apply_max_threads)(int coef);
-  // mode: MODE_PLAIN or MODE_PCG; args points to PrecArgsT<T>
-  cudaError_t (*precond)(int mode, const void *args, int n_items, int threads, cudaStream_t s);
+  // mode: MODE_PLAIN or MODE_PCG; args points to PrecArgsT<T>; sms: SMs of the device
+  cudaError_t (*precond)(int mode, const void *args, int n_items, int sms, cudaStream_t s);
   // volume transpose in integration-by-parts form (COEF_LAPLACE, COEF_SCALAR;
   // args as for MODE_TRANSPOSE); ibp_smem: its shared memory, 0 where the
   // instance is not built
