@@ -48,10 +48,10 @@ def _generate():
                 with open(path, "w") as f:
                     f.write(text)
             units.append(path)
-    # second FP64 launch shape of the apply kernels (threads per CTA, see csrc/registry.h)
-    for w, nt in ((2, 128), (3, 128), (4, 192), (5, 256), (6, 128), (7, 128)):
+    # second FP64 launch shape of the apply kernels (ALT_W0 to ALT_W1 of csrc/registry.h)
+    for w in range(2, 8):
         path = os.path.join(GEN, f"inst_f64b_w{w}.cu")
-        text = (f"#define REAL double\n#define WDEG {w}\n#define HPSE_APPLY_NT {nt}\n#define HPSE_LINES_NC 4\n"
+        text = (f"#define REAL double\n#define WDEG {w}\n#define HPSE_LINES_NC 4\n"
                 f"#define HPSE_APPLY_ONLY\n#define HPSE_REGISTER_NAME hpse_register_f64b_w{w}\n#define HPSE_DOUBLE\n"
                 f'#include "inst_template.cuh"\n')
         if not os.path.exists(path) or open(path).read() != text:

@@ -16,7 +16,8 @@
 // four]: a thread per row reads its row in coalesced 16-byte loads.
 //
 // One CTA (4 warps) per (element, 128-row tile, 64 right-hand sides), four CTAs
-// to an SM: K in chunks of 32, BJT_STAGES stages.  A (128 rows, hi and lo) goes
+// to an SM: K in chunks of 32, one stage (with three stages and two CTAs 578 us for
+// 368: too few warps for the load latency).  A (128 rows, hi and lo) goes
 // from registers to tensor memory (tcgen05.st, thread = row = lane), which the
 // MMA reads as its A operand: held in shared memory, hi and lo took 32 KB of
 // writes and 48 KB of operand reads per chunk (535 us for 512 blocks of 729 at
@@ -41,16 +42,11 @@ constexpr int BJT_K = 32;                // K per stage: one 128-byte row of FP3
 constexpr int BJT_THREADS = 128;
 constexpr int BJT_B_BYTES = BJT_N * BJT_K * 4;  // 8 KB
 constexpr int BJT_STAGE_BYTES = 2 * BJT_B_BYTES;
-#if defined(HPSE_BJT_STAGES)
-constexpr int BJT_STAGES = HPSE_BJT_STAGES;  // set at build time (pipeline-depth experiments)
-#else
-constexpr int BJT_STAGES = 1;  // 4 CTAs per SM hide more load latency than 3 stages and 2 CTAs (368 and 578 us)
-#endif
-// tensor memory: accumulator (64 columns), then per stage A hi and A lo (32 columns each)
-constexpr int BJT_TMEM_COLS = BJT_STAGES == 1 ? 128 : 256;
+// tensor memory: accumulator (64 columns), A hi and A lo (32 columns each)
+constexpr int BJT_TMEM_COLS = 128;
 constexpr int BJT_MINB = 512 / BJT_TMEM_COLS;  // CTAs per SM that the tensor memory allows
-constexpr size_t BJT_SMEM = BJT_STAGES * (size_t)BJT_STAGE_BYTES + 1024;  // stages + alignment slack
-static_assert(BJT_N + BJT_STAGES * 2 * BJT_K <= BJT_TMEM_COLS, "tensor memory");
+constexpr size_t BJT_SMEM = (size_t)BJT_STAGE_BYTES + 1024;  // the stage + alignment slack
+static_assert(BJT_N + 2 * BJT_K <= BJT_TMEM_COLS, "tensor memory");
 constexpr int BJT_TILE = BJT * BJT;      // floats per tile
 
 // tiles per copy (X or X^T) of an n x n factor
@@ -132,7 +128,7 @@ __device__ __forceinline__ bool bjt_wait(uint32_t bar, uint32_t parity, int poll
 template <bool TRANS>
 __global__ void __launch_bounds__(BJT_THREADS, BJT_MINB) k_bj_tc(BjTcArgs A, const float *Xt, const float *in, float *out) {
   extern __shared__ unsigned char bjt_raw[];
-  __shared__ __align__(8) uint64_t bar[BJT_STAGES];
+  __shared__ __align__(8) uint64_t bar;
   __shared__ uint32_t s_tmem;
   __shared__ int s_bad;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -145,7 +141,7 @@ __global__ void __launch_bounds__(BJT_THREADS, BJT_MINB) k_bj_tc(BjTcArgs A, con
   const int64_t vb = A.dof_off[e];
   const int nblk = bjt_blocks(n);
   const float *tiles = Xt + A.tile_off[e] + (TRANS ? (int64_t)nblk * BJT_TILE : 0);
-  // stage buffers on a 1024-byte boundary
+  // the stage on a 1024-byte boundary
   const uint32_t raw = bjt_smem(bjt_raw);
   unsigned char *sm = bjt_raw + (((raw + 1023u) & ~1023u) - raw);
   const uint32_t sbase = bjt_smem(sm);
@@ -161,8 +157,7 @@ __global__ void __launch_bounds__(BJT_THREADS, BJT_MINB) k_bj_tc(BjTcArgs A, con
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   if (tid == 0) {
-    for (int i = 0; i < BJT_STAGES; ++i)
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bjt_smem(&bar[i])) : "memory");
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bjt_smem(&bar)) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     s_bad = 0;
   }
@@ -196,10 +191,10 @@ __global__ void __launch_bounds__(BJT_THREADS, BJT_MINB) k_bj_tc(BjTcArgs A, con
       for (int j = 0; j < 16; ++j, src += A.ndof) rb[j] = j < m ? *src : 0.0f;
     }
   };
-  auto store = [&](int st) {
-    unsigned char *sb_hi = sm + st * BJT_STAGE_BYTES, *sb_lo = sb_hi + BJT_B_BYTES;
+  auto store = [&]() {
+    unsigned char *sb_hi = sm, *sb_lo = sb_hi + BJT_B_BYTES;
     // the warp's 32 lanes of tensor memory: its 32 rows of the tile
-    const uint32_t ta = tmem + ((uint32_t)(32 * warp) << 16) + BJT_N + st * 2 * BJT_K;
+    const uint32_t ta = tmem + ((uint32_t)(32 * warp) << 16) + BJT_N;
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
       float h[16], l[16];
@@ -232,14 +227,13 @@ __global__ void __launch_bounds__(BJT_THREADS, BJT_MINB) k_bj_tc(BjTcArgs A, con
   load(kc0);
   int last = -1;
   for (int kc = kc0; kc < kc1; ++kc) {
-    const int it = kc - kc0, st = it % BJT_STAGES;
-    // the MMAs that last read this stage (iteration it - BJT_STAGES) are done
-    if (it >= BJT_STAGES && tid == 0 && !bjt_wait(bjt_smem(&bar[st]), ((it - BJT_STAGES) / BJT_STAGES) & 1, A.polls))
-      s_bad = 1;
+    const int it = kc - kc0;
+    // the MMAs of the chunk before are done with the stage
+    if (it >= 1 && tid == 0 && !bjt_wait(bjt_smem(&bar), (it - 1) & 1, A.polls)) s_bad = 1;
     __syncthreads();
     if (s_bad) break;
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    store(st);
+    store();
     asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -247,8 +241,8 @@ __global__ void __launch_bounds__(BJT_THREADS, BJT_MINB) k_bj_tc(BjTcArgs A, con
     if (kc + 1 < kc1) load(kc + 1);
     if (tid == 0) {
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint32_t a_hi = tmem + BJT_N + st * 2 * BJT_K, a_lo = a_hi + BJT_K;
-      const uint32_t b_hi = sbase + st * BJT_STAGE_BYTES, b_lo = b_hi + BJT_B_BYTES;
+      const uint32_t a_hi = tmem + BJT_N, a_lo = a_hi + BJT_K;
+      const uint32_t b_hi = sbase, b_lo = b_hi + BJT_B_BYTES;
 #pragma unroll
       for (int s = 0; s < 4; ++s) {
         // K-step s: 8 TF32, 8 columns of A and 32 bytes further along the swizzled rows of B
@@ -267,7 +261,7 @@ __global__ void __launch_bounds__(BJT_THREADS, BJT_MINB) k_bj_tc(BjTcArgs A, con
         }
       }
       asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                       bjt_smem(&bar[st]))
+                       bjt_smem(&bar))
                    : "memory");
     }
     last = it;
@@ -275,10 +269,9 @@ __global__ void __launch_bounds__(BJT_THREADS, BJT_MINB) k_bj_tc(BjTcArgs A, con
   // the last commit covers every MMA issued before it; after an expired wait the MMAs
   // in flight end (bounded) before the tensor memory is freed
   if (tid == 0 && last >= 0) {
-    const uint32_t mb = bjt_smem(&bar[last % BJT_STAGES]), par = (last / BJT_STAGES) & 1;
-    if (s_bad || !bjt_wait(mb, par, A.polls)) {
+    if (s_bad || !bjt_wait(bjt_smem(&bar), last & 1, A.polls)) {
       s_bad = 1;
-      bjt_wait(mb, par, BJ_POLLS);
+      bjt_wait(bjt_smem(&bar), last & 1, BJ_POLLS);
     }
   }
   __syncthreads();

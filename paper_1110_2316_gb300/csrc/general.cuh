@@ -46,11 +46,7 @@ namespace {
 
 constexpr int GEN_NC = 12;
 // resident CTAs asked for: about 20 warps per SM in FP32 (96 registers at W = 8)
-#if defined(HPSE_GEN_MINB)
-constexpr int GEN_MINB = HPSE_GEN_MINB;  // set at build time (launch-shape experiments)
-#else
 constexpr int GEN_MINB = sizeof(real) == 8 ? 1 : (640 / NT < 1 ? 1 : (640 / NT > 4 ? 4 : 640 / NT));
-#endif
 
 struct GenLayout {
   static constexpr int TS = t_stride(3, 6, GEN_MINB);  // row stride of the T fields

@@ -73,6 +73,7 @@ static void init_registry() {
   }
   const RegFn alt[] = {hpse_register_f64b_w2, hpse_register_f64b_w3, hpse_register_f64b_w4,
                        hpse_register_f64b_w5, hpse_register_f64b_w6, hpse_register_f64b_w7};
+  static_assert(sizeof(alt) / sizeof(alt[0]) == hpse::ALT_W1 - hpse::ALT_W0 + 1, "units of the second launch shape");
   for (int w = hpse::ALT_W0; w <= hpse::ALT_W1; ++w) alt[w - hpse::ALT_W0](&g_alt[w]);
   g_sets_ready = true;
 }
@@ -3958,46 +3959,41 @@ extern "C" hpse_status hpse_h1_error(hpse_mesh *m, const double *u, const double
 //   dJ/d(d_k a) = w J [d_k u L lambda + (L u - f) d_k lambda]
 // (differentiate -lambda^T sum_q z_q dz_q/du with respect to each datum).
 // ---------------------------------------------------------------------------
-template <typename T>
-struct FieldArgsT {
+struct FieldArgs {
   int n_rhs;
   int64_t ndof, nquad;
   const int64_t *dof_off, *coef_off;
   const int32_t *elem_W;
   const double *geo;
   const double *const *qtab;  // per degree: B0, B1 (QxP), DQ, KQ (QxQ), wq (Q), B2 (QxP)
-  const T *u;
-  T *out;                     // [n_rhs][5][nquad]
+  const double *u;
+  double *out;                // [n_rhs][5][nquad]
 };
-typedef FieldArgsT<double> FieldArgs;
 
 // (v, v_x, v_y, v_z, Lap v) of a DOF vector at the volume points; one block per (element, rhs)
-// point fields in the precision T (FP64 tables rounded to T)
-template <typename T>
-__global__ void k_fields(FieldArgsT<T> A) {
-  extern __shared__ __align__(16) unsigned char fields_raw[];
-  T *sm = reinterpret_cast<T *>(fields_raw);
+__global__ void k_fields(FieldArgs A) {
+  extern __shared__ double sm[];
   const int item = blockIdx.x;
   const int e = item / A.n_rhs, r = item - e * A.n_rhs;
   const int W = A.elem_W[e], P = W + 1, Q = 2 * W + 1;
   const double *tb = A.qtab[W];
   const double *B0 = tb, *B1 = tb + Q * P, *B2 = tb + 2 * Q * P + 2 * Q * Q + Q;
   const double *geo = A.geo + (int64_t)e * 4;
-  const T sx = (T)geo[0], sy = (T)geo[1], sz = (T)geo[2];
-  T *blk = sm, *X0 = blk + P * P * P, *X1 = X0 + Q * P * P, *X2 = X1 + Q * P * P;
-  T *Ta = X2 + Q * P * P, *Tb = Ta + Q * Q * P, *Tc = Tb + Q * Q * P;
+  const double sx = geo[0], sy = geo[1], sz = geo[2];
+  double *blk = sm, *X0 = blk + P * P * P, *X1 = X0 + Q * P * P, *X2 = X1 + Q * P * P;
+  double *Ta = X2 + Q * P * P, *Tb = Ta + Q * Q * P, *Tc = Tb + Q * Q * P;
   const int64_t base = (int64_t)r * A.ndof + A.dof_off[e];
   const int nt = blockDim.x;
   for (int t = threadIdx.x; t < P * P * P; t += nt) blk[t] = A.u[base + t];
   __syncthreads();
   for (int t = threadIdx.x; t < Q * P * P; t += nt) {
     const int qa = t % Q, l = t / Q;
-    T a0 = 0, a1 = 0.0, a2 = 0.0;
+    double a0 = 0, a1 = 0.0, a2 = 0.0;
     for (int i = 0; i < P; ++i) {
-      const T v = blk[l * P + i];
-      a0 += (T)B0[qa * P + i] * v;
-      a1 += (T)B1[qa * P + i] * v;
-      a2 += (T)B2[qa * P + i] * v;
+      const double v = blk[l * P + i];
+      a0 += B0[qa * P + i] * v;
+      a1 += B1[qa * P + i] * v;
+      a2 += B2[qa * P + i] * v;
     }
     X0[l * Q + qa] = a0;
     X1[l * Q + qa] = a1;
@@ -4007,12 +4003,12 @@ __global__ void k_fields(FieldArgsT<T> A) {
   // pass A: T_a = B0y X0, T_b = B1y X0, T_c = B0y X1
   for (int t = threadIdx.x; t < Q * Q * P; t += nt) {
     const int qa = t % Q, qb = (t / Q) % Q, k = t / (Q * Q);
-    T a = 0, b = 0.0, c = 0.0;
+    double a = 0, b = 0.0, c = 0.0;
     for (int j = 0; j < P; ++j) {
-      const T x0 = X0[(k * P + j) * Q + qa];
-      a += (T)B0[qb * P + j] * x0;
-      b += (T)B1[qb * P + j] * x0;
-      c += (T)B0[qb * P + j] * X1[(k * P + j) * Q + qa];
+      const double x0 = X0[(k * P + j) * Q + qa];
+      a += B0[qb * P + j] * x0;
+      b += B1[qb * P + j] * x0;
+      c += B0[qb * P + j] * X1[(k * P + j) * Q + qa];
     }
     Ta[t] = a;
     Tb[t] = b;
@@ -4022,14 +4018,14 @@ __global__ void k_fields(FieldArgsT<T> A) {
   const int64_t ob = (int64_t)r * 5 * A.nquad + A.coef_off[e];
   for (int t = threadIdx.x; t < Q * Q * Q; t += nt) {
     const int qa = t % Q, qb = (t / Q) % Q, qc = t / (Q * Q);
-    T v = 0, vz = 0.0, vzz = 0.0, vy = 0.0, vx = 0.0;
+    double v = 0, vz = 0.0, vzz = 0.0, vy = 0.0, vx = 0.0;
     for (int k = 0; k < P; ++k) {
       const int o = (k * Q + qb) * Q + qa;
-      v += (T)B0[qc * P + k] * Ta[o];
-      vz += (T)B1[qc * P + k] * Ta[o];
-      vzz += (T)B2[qc * P + k] * Ta[o];
-      vy += (T)B0[qc * P + k] * Tb[o];
-      vx += (T)B0[qc * P + k] * Tc[o];
+      v += B0[qc * P + k] * Ta[o];
+      vz += B1[qc * P + k] * Ta[o];
+      vzz += B2[qc * P + k] * Ta[o];
+      vy += B0[qc * P + k] * Tb[o];
+      vx += B0[qc * P + k] * Tc[o];
     }
     A.out[ob + t] = v;
     A.out[ob + A.nquad + t] = sx * vx;
@@ -4041,10 +4037,10 @@ __global__ void k_fields(FieldArgsT<T> A) {
   // pass B: T_a = B2y X0 (u_yy), T_b = B0y X2 (u_xx)
   for (int t = threadIdx.x; t < Q * Q * P; t += nt) {
     const int qa = t % Q, qb = (t / Q) % Q, k = t / (Q * Q);
-    T a = 0, b = 0.0;
+    double a = 0, b = 0.0;
     for (int j = 0; j < P; ++j) {
-      a += (T)B2[qb * P + j] * X0[(k * P + j) * Q + qa];
-      b += (T)B0[qb * P + j] * X2[(k * P + j) * Q + qa];
+      a += B2[qb * P + j] * X0[(k * P + j) * Q + qa];
+      b += B0[qb * P + j] * X2[(k * P + j) * Q + qa];
     }
     Ta[t] = a;
     Tb[t] = b;
@@ -4052,11 +4048,11 @@ __global__ void k_fields(FieldArgsT<T> A) {
   __syncthreads();
   for (int t = threadIdx.x; t < Q * Q * Q; t += nt) {
     const int qa = t % Q, qb = (t / Q) % Q, qc = t / (Q * Q);
-    T vyy = 0, vxx = 0.0;
+    double vyy = 0, vxx = 0.0;
     for (int k = 0; k < P; ++k) {
       const int o = (k * Q + qb) * Q + qa;
-      vyy += (T)B0[qc * P + k] * Ta[o];
-      vxx += (T)B0[qc * P + k] * Tb[o];
+      vyy += B0[qc * P + k] * Ta[o];
+      vxx += B0[qc * P + k] * Tb[o];
     }
     A.out[ob + 4 * A.nquad + t] += sy * sy * vyy + sx * sx * vxx;
   }
@@ -4220,9 +4216,8 @@ __global__ void k_data_grad_vjp(int64_t nquad, int n_rhs, const double *aux, con
   }
 }
 
-template <typename T = double>
-static FieldArgsT<T> field_args(const hpse_mesh *m, const T *u, T *out) {
-  FieldArgsT<T> A;
+static FieldArgs field_args(const hpse_mesh *m, const double *u, double *out) {
+  FieldArgs A;
   A.n_rhs = m->n_rhs;
   A.ndof = m->ndof;
   A.nquad = m->nquad;
@@ -4242,12 +4237,11 @@ static int max_degree(const hpse_mesh *m) {
   return w;
 }
 
-template <typename T = double>
-static hpse_status launch_fields(hpse_mesh *m, const T *u, T *out, cudaStream_t s) {
+static hpse_status launch_fields(hpse_mesh *m, const double *u, double *out, cudaStream_t s) {
   const int W = max_degree(m), P = W + 1, Q = 2 * W + 1;
-  const size_t smem = (size_t)(P * P * P + 3 * Q * P * P + 3 * Q * Q * P) * sizeof(T);
-  CK(raise_smem((const void *)k_fields<T>, m->device, (size_t)smem));
-  k_fields<T><<<n_items_all(m), 256, smem, s>>>(field_args<T>(m, u, out));
+  const size_t smem = (size_t)(P * P * P + 3 * Q * P * P + 3 * Q * Q * P) * sizeof(double);
+  CK(raise_smem((const void *)k_fields, m->device, (size_t)smem));
+  k_fields<<<n_items_all(m), 256, smem, s>>>(field_args(m, u, out));
   CK(cudaGetLastError());
   ++g_launches;
   return HPSE_OK;
@@ -4275,7 +4269,7 @@ extern "C" hpse_status hpse_apply_eval_transpose(hpse_mesh *m, const double *rho
   const int W = max_degree(m), P = W + 1, Q = 2 * W + 1;
   const size_t smem = (size_t)(Q * Q * Q + Q * Q * P + Q * P * P) * sizeof(double);
   CK(raise_smem((const void *)k_eval_T, m->device, (size_t)smem));
-  k_eval_T<<<n_items_all(m), 256, smem, (cudaStream_t)stream>>>(field_args<double>(m, nullptr, y), rho);
+  k_eval_T<<<n_items_all(m), 256, smem, (cudaStream_t)stream>>>(field_args(m, nullptr, y), rho);
   CK(cudaGetLastError());
   ++g_launches;
   return HPSE_OK;
@@ -4292,7 +4286,7 @@ extern "C" hpse_status hpse_apply_fields_transpose(hpse_mesh *m, const double *w
   const int W = max_degree(m), P = W + 1, Q = 2 * W + 1;
   const size_t smem = (size_t)(Q * Q * Q + Q * Q * P + Q * P * P + P * P * P) * sizeof(double);
   CK(raise_smem((const void *)k_fields_T, m->device, (size_t)smem));
-  k_fields_T<<<n_items_all(m), 256, smem, (cudaStream_t)stream>>>(field_args<double>(m, nullptr, y), wf);
+  k_fields_T<<<n_items_all(m), 256, smem, (cudaStream_t)stream>>>(field_args(m, nullptr, y), wf);
   CK(cudaGetLastError());
   ++g_launches;
   return HPSE_OK;

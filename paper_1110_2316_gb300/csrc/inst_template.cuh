@@ -1,8 +1,8 @@
 // inst_template.cuh -- launchers for one (REAL, WDEG) instantiation of
 // kernels.cuh.  A generated translation unit defines REAL, WDEG,
 // HPSE_REGISTER_NAME (and HPSE_DOUBLE for REAL = double), then includes this.
-// HPSE_APPLY_ONLY with HPSE_APPLY_NT, HPSE_LINES_NC: the apply kernels alone in a
-// second launch shape.
+// HPSE_APPLY_ONLY with HPSE_LINES_NC: the apply kernels alone in a second launch
+// shape (registry.h).
 #include <vector>
 
 #include "kernels.cuh"

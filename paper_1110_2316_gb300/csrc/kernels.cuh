@@ -84,8 +84,9 @@ __host__ __device__ constexpr bool odd_pp(int t) { return t < 2; }
 #endif
 #define PAD32(n) ((((n) + 31) / 32) * 32)
 constexpr int NT_RAW = PAD32(Q2);
-#if defined(HPSE_APPLY_NT)
-constexpr int NT = HPSE_APPLY_NT;  // set by the unit (second FP64 launch shape, see registry.h)
+#if defined(HPSE_APPLY_ONLY)
+static_assert(WDEG >= hpse::ALT_W0 && WDEG <= hpse::ALT_W1, "degrees of the second launch shape");
+constexpr int NT = hpse::ALT_THREADS[WDEG - hpse::ALT_W0];  // second FP64 launch shape
 #else
 constexpr int NT = NT_RAW < 64 ? 64 : (NT_RAW > HPSE_APPLY_MAXT ? HPSE_APPLY_MAXT : NT_RAW);
 #endif
@@ -234,7 +235,7 @@ struct Lines {
   static constexpr int PADL = PAD32(L);
   static constexpr int NC_RAW = NT / PADL;
 #if defined(HPSE_LINES_NC)
-  static constexpr int NC_MAX = HPSE_LINES_NC;  // set by the unit, with HPSE_APPLY_NT
+  static constexpr int NC_MAX = HPSE_LINES_NC;  // set by the unit, with HPSE_APPLY_ONLY
 #else
   static constexpr int NC_MAX = 2;
 #endif
@@ -1301,11 +1302,7 @@ struct ApplyLayout {
   static constexpr bool RHO_FITS =
       ((size_t)(TOTAL0 + RHO_LEN) * sizeof(real) + 64 * sizeof(double) + 1024) * APPLY_MINB <= 232448;
   static constexpr bool RHO_INPLACE = sizeof(real) == 4 || !RHO_FITS;
-#if defined(HPSE_APPLY_RHO_REG)
-  static constexpr bool RHO_SMEM = false;  // set at build time (layout experiments)
-#else
   static constexpr bool RHO_SMEM = !RHO_INPLACE && RHO_FITS;
-#endif
   static constexpr int TOTAL = TOTAL0 + (RHO_SMEM ? RHO_LEN : 0);
   // the FP64 reduction buffer starts on a 16-byte boundary whatever REAL is
   static constexpr size_t END = (((size_t)TOTAL * sizeof(real) + 15) / 16) * 16;

@@ -133,6 +133,7 @@ inline int packed_table_size(int W) {
 // other (1,024 items: W = 6 387 -> 346 / 605 -> 564 us, W = 7 537 -> 503 / 887 ->
 // 843); a lone item is slower (57.6 -> 65.7 us).
 constexpr int ALT_W0 = 2, ALT_W1 = 7;
+constexpr int ALT_THREADS[ALT_W1 - ALT_W0 + 1] = {128, 128, 192, 256, 128, 128};
 inline bool alt_shape(int W, long long items, long long all_items, int sms) {
   if (W < ALT_W0 || W > ALT_W1) return false;
   return W <= 5 ? all_items <= sms : items > sms;  // all_items: over every degree of the launch
