@@ -343,13 +343,16 @@ hpse_status hpse_setup_block_preconditioner(hpse_mesh *m);
  * just built (variants 0-2 and 8 for >= 32 right-hand sides, 3-4 for 2..31,
  * 5-7 for one; 2, 4, 6 and 8 in FP32 only) and keeps the fastest.  Variants
  * 2, 4 and 6 in FP32 and 3 and 5 in FP64 take both products in one pass over
- * the factor, the others of 0-7 are CUDA-core tiles; variant 8 runs both products on the
+ * the factor; for blocks of W >= 6 and five or more right-hand sides the FP32
+ * ones split each operand into two TF32 parts, as variant 8 does, in sums of 16
+ * terms (error 1.6e-7 against 64 bits at W = 8, FP32 multiply-adds 3e-7; a
+ * right-hand side that is below 2^-110 throughout loses digits).  The others of
+ * 0-7 are CUDA-core tiles; variant 8 runs both products on the
  * tensor cores (tcgen05, 128 rows x 64 right-hand sides per CTA, each FP32
  * operand split into two TF32 parts, three MMAs per product, FP32
  * accumulation in tensor memory).  hpse_block_tile returns the chosen
- * variant, its tile (rows x right-hand sides per CTA; a one-pass variant works on all
- * (W+1)^3 rows of a block) and, if ms is not NULL,
- * the measured milliseconds of each of the 9 variants (0 for those not tried);
+ * variant, its tile (rows x right-hand sides per CTA; a one-pass variant works
+ * on all (W+1)^3 rows of a block) and, if ms is not NULL, the measured milliseconds of each of the 9 variants (0 for those not tried);
  * HPSE_ERR_NO_DATA before the set-up.  hpse_set_block_tile overrides the
  * choice (HPSE_ERR_INVALID_ARG for a variant that does not exist in that
  * precision, or variant 8 when its tiles were not built).  No counterpart in

@@ -1,6 +1,7 @@
 // bj_pass.cuh -- z = X^T (X r) of the element-block preconditioner in ONE pass
-// over the packed factor X (block_precond.cuh): FP64 for any right-hand-side
-// count below 32, FP32 for up to 4 (bj_mma.cuh takes 5 to 31).
+// over the packed factor X (block_precond.cuh): the one-pass variants in FP64,
+// and in FP32 for up to 4 right-hand sides and for blocks up to n = 256 at any
+// count (bj_mma.cuh takes the others, bj_pass.cu).
 //
 // The two products of k_bj_tri read X twice and keep a multiply-add per shared
 // load; at few right-hand sides the apply is bound by those reads.  Here a CTA
@@ -17,7 +18,8 @@
 // a cluster of up to 8 CTAs shares one: row blocks are dealt in turn and the
 // partial z summed through distributed shared memory in rank order.
 // Bound: FP32 HBM (the factor once: 545 MB for 512 blocks of 729, 80 us; 145 us
-// at 1 and 215 us at 4 right-hand sides, issue-limited), FP64 its pipe (two
+// at 1 and 215 us at 4 right-hand sides: latency of the copies, sums and barriers
+// at twelve warps per SM, no pipe above 25 %), FP64 its pipe (two
 // lanes per clock and SM: 1.73 ms at 4 right-hand sides, 2.42 ms measured).
 // Waits on the copies are bounded (bj_pass.h).
 #pragma once

@@ -34,8 +34,9 @@
 // in two sweeps (lines T02, T10, T11, T20, then T00, T01, whose slots rho
 // occupies).  Field by field with rho in registers the forward spilled 1.5 KB
 // per thread and loaded each coefficient alone at a 48-byte lane stride.
-// Bound: FP32 the packed FMAs and the coefficient reads from L2 (48 bytes per
-// point, twice per apply), FP64 its pipe.  8^3 elements of W = 8: FP32, 16 rhs
+// Bound: FP32 the latency of the coefficient reads from L2 (12, 8 and 12 values
+// of a point in the three sweeps: 128 bytes; long-scoreboard 5.4 stalls per
+// issue, no pipe above 26 %) at two CTAs per SM, FP64 its pipe.  8^3 elements of W = 8: FP32, 16 rhs
 // 2394 -> 895 us; FP64, 2 rhs 2979 -> 2463 us.  Shared memory: su | X[3] | T[6] |
 // D copy + face scales | reduction; the T region later holds sy and the face
 // scratch.  Instances whose layout exceeds 227 KB (FP64 at W = 10) are not
