@@ -340,8 +340,9 @@ hpse_status hpse_setup_block_preconditioner(hpse_mesh *m);
 /* Tile shape of the element-block preconditioner's two triangular products,
  * per degree W and precision: hpse_setup_block_preconditioner times every
  * candidate shape for the mesh's right-hand-side count on the factors it has
- * just built (variants 0-2 and 8 for >= 32 right-hand sides, 3-4 for 2..31,
- * 5-7 for one; 2, 4, 6 and 8 in FP32 only) and keeps the fastest.  Variants
+ * just built (variants 0-2 and 8 for >= 32 right-hand sides, 3-4 for 2..31 [in
+ * FP64 4 on many large blocks only], 5-7 for one; 2 and 8 in FP32 only) and keeps
+ * the fastest.  Variants
  * 2, 4 and 6 in FP32 and 3 and 5 in FP64 take both products in one pass over
  * the factor; for blocks of W >= 6 and five or more right-hand sides the FP32
  * ones split each operand into two TF32 parts, as variant 8 does, in sums of 16

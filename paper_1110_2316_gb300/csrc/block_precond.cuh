@@ -429,27 +429,30 @@ __global__ void __launch_bounds__(32 * BJ_VEC_ITEMS) k_bj_dot(BjArgs A, const T 
 // (bj_pass.cuh, bj_mma.cuh); the other variants below 8 are tiles of k_bj_tri
 // (rows x right-hand sides per CTA), variant 8 is the tensor-core form
 // (bj_tc.cuh: 128 rows x 64 right-hand sides, 3xTF32), offered from 32
-// right-hand sides on.  Variants 2, 4, 6 and 8 exist in FP32 only.
+// right-hand sides on.  Variants 2 and 8 exist in FP32 only.
 // 512 factors of n = 729, one application, tiles -> pass:
 // FP32 270 -> 145 us (1 rhs), 468 -> 215 (4), 470 -> 242 (8), 871 -> 359 (16);
 // FP64 4820 -> 2417 us (4), 4810 -> 4600 (8), and for 8 blocks 400 -> 98 us
-// (4).  One FP64 right-hand side of many blocks stays with the 64 x 1 tile
-// (622 us against 767), of few blocks the pass is the faster (41 against 89).
+// (4).  In FP64 many large blocks can be faster as tiles (128 blocks of n = 1000:
+// 12 rhs 4506, 4805 us in one pass; one rhs 390 and 411), whose FP64 work is the
+// same: there the 128 x 8 tile is timed beside the pass, from n = 729 and half the
+// SMs on (32 blocks: 1786, 1198 in one pass), and two tiles at one right-hand side.
 constexpr int BJ_NVAR = 9;
 constexpr int BJ_TC = 8;
-constexpr int BJ_TILE[BJ_NVAR][2] = {{64, 64}, {128, 32}, {256, 16}, {128, 8}, {256, 8},
-                                     {128, 1}, {256, 1},  {64, 1},   {128, 64}};
+// (an entry of a one-pass variant serves the other precision's tile)
+constexpr int BJ_TILE[BJ_NVAR][2] = {{64, 64}, {128, 32}, {0, 0},  {128, 8}, {128, 8},
+                                     {128, 1}, {128, 1},  {64, 1}, {128, 64}};
 inline bool bj_is_pass(int v, bool fp32) { return fp32 ? (v == 2 || v == 4 || v == 6) : (v == 3 || v == 5); }
-inline bool bj_variant_ok(int v, bool fp32) {
-  return v >= 0 && v < BJ_NVAR && (fp32 || (v != 2 && v != 4 && v != 6 && v != BJ_TC));
-}
-inline int bj_candidates(int n_rhs, bool fp32, int *v) {
-  int n = 0;
+inline bool bj_variant_ok(int v, bool fp32) { return v >= 0 && v < BJ_NVAR && (fp32 || (v != 2 && v != BJ_TC)); }
+// candidates for n_group blocks of size n
+inline int bj_candidates(int n, int n_group, int n_rhs, int sms, bool fp32, int *v) {
+  int c = 0;
   const int all[3][4] = {{0, 1, 2, BJ_TC}, {3, 4, -1, -1}, {5, 6, 7, -1}};
-  const int *c = all[n_rhs >= 32 ? 0 : (n_rhs >= 2 ? 1 : 2)];
+  const int *a = all[n_rhs >= 32 ? 0 : (n_rhs >= 2 ? 1 : 2)];
+  const bool tile = fp32 || (n_rhs >= 9 && n >= 729 && 2 * n_group >= sms);
   for (int i = 0; i < 4; ++i)
-    if (c[i] >= 0 && bj_variant_ok(c[i], fp32)) v[n++] = c[i];
-  return n;
+    if (a[i] >= 0 && bj_variant_ok(a[i], fp32) && (a[i] != 4 || tile)) v[c++] = a[i];
+  return c;
 }
 
 template <typename T, int TM, int RT, int TR, int TC>
@@ -466,12 +469,8 @@ static cudaError_t bj_apply_group(const BjArgs &a, const T *X, const T *r, T *t,
   if (v == 0) bj_pair<T, 64, 64, 16, 16>(a, X, r, t, z, s);
   else if (v == 1) bj_pair<T, 128, 32, 32, 8>(a, X, r, t, z, s);
   else if (v == 7) bj_pair<T, 64, 1, 64, 1>(a, X, r, t, z, s);
-  else if constexpr (sizeof(T) == 4) {
-    if (v == 3) bj_pair<T, 128, 8, 64, 4>(a, X, r, t, z, s);
-    else if (v == 5) bj_pair<T, 128, 1, 128, 1>(a, X, r, t, z, s);
-    else return cudaErrorInvalidValue;
-  } else {
-    return cudaErrorInvalidValue;
-  }
+  else if (v == (sizeof(T) == 4 ? 3 : 4)) bj_pair<T, 128, 8, 64, 4>(a, X, r, t, z, s);
+  else if (v == (sizeof(T) == 4 ? 5 : 6)) bj_pair<T, 128, 1, 128, 1>(a, X, r, t, z, s);
+  else return cudaErrorInvalidValue;
   return cudaGetLastError();
 }

@@ -3130,7 +3130,7 @@ extern "C" hpse_status hpse_setup_block_preconditioner(hpse_mesh *m) {
       const BjArgs ba = bj_args(m, g, m->n_rhs);
       for (int pi = 0; pi < 2; ++pi) {
         int cand[4];
-        const int nc2 = bj_candidates(m->n_rhs, pi == 1, cand);
+        const int nc2 = bj_candidates(ba.n, g.n, m->n_rhs, m->n_sm, pi == 1, cand);
         float best = 1e30f;
         for (int k = 0; k < BJ_NVAR; ++k) m->bj_ms[g.W][pi][k] = 0.0f;
         m->bj_var[g.W][pi] = 0;  // a tile of both precisions and any count, if no candidate is left
