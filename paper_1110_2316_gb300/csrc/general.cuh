@@ -37,7 +37,9 @@
 // Bound: FP32 the latency of the coefficient reads from L2 (12, 8 and 12 values
 // of a point in the three sweeps: 128 bytes; long-scoreboard 5.4 stalls per
 // issue, no pipe above 26 %) at two CTAs per SM, FP64 its pipe.  8^3 elements of W = 8: FP32, 16 rhs
-// 2394 -> 895 us; FP64, 2 rhs 2979 -> 2463 us.  Shared memory: su | X[3] | T[6] |
+// 2394 -> 895 us; FP64, 2 rhs 2979 -> 2463 us.  (FP64 at W = 1, four lines and nine
+// columns, is slower than field by field: 240 items 18.5 -> 20.5 us, 8,192 items
+// 225 -> 231; its coefficients kept in registers gave 20.4 and 236.)  Shared memory: su | X[3] | T[6] |
 // D copy + face scales | reduction; the T region later holds sy and the face
 // scratch.  Instances whose layout exceeds 227 KB (FP64 at W = 10) are not
 // built; the host library refuses such meshes.

@@ -1009,7 +1009,19 @@ __device__ void face_phase(const ApplyArgs &A, int e, int r, const real *su, rea
       if (!job(t, kind, fld, f, ln)) continue;
       const int ob = fld == 2 ? ln : ln * P, os = fld == 2 ? P : 1;
       real ev[HPE], od[HPE], al[P], be[P];
-      if (kind == 2) {
+      if (W == 1 && kind != 0) {
+        // a warp holds every field here: fields 0 and 3 share what they can (FP64, 80
+        // items: branches of their own 15.5 us, so 14.5)
+        load_fold(FSLOT(f, fld ? sJ3 : sJ0) + ob, os, ev, od);
+        if (fld == 0) {
+          pp_line<2>(ev, od, al);
+#pragma unroll
+          for (int i = 0; i < P; ++i) be[i] = (real)0;
+        } else {
+          pp_line<4>(ev, od, al);
+          pp_line<2>(ev, od, be);
+        }
+      } else if (kind == 2) {
         load_fold(FSLOT(f, sJ0) + ob, os, ev, od);
         pp_line<2>(ev, od, al);
       } else if (kind == 1) {
@@ -1047,7 +1059,7 @@ __device__ void face_phase(const ApplyArgs &A, int e, int r, const real *su, rea
 #pragma unroll
       for (int i = 0; i < P; ++i) {
         Bs[i * os] = al[i];
-        if (kind != 2) As[i * os] = be[i];
+        if (W == 1 || kind != 2) As[i * os] = be[i];
       }
     }
     __syncthreads();
