@@ -28,9 +28,8 @@ def test_tile_of_the_variants(W, n_rhs, f32, f64):
                                                  ((2, 1, 1), 1, True)])
 def test_fp64_tiles_beside_the_pass(boxes, n_rhs, offered):
     # many large blocks can be faster as tiles in FP64 (128 rows x 8 right-hand sides, 128 x 1):
-    # they are timed there, and give the products of the one-pass variant (two sums of n terms
-    # each: 4 n eps |X|^T |X| |r|, here with |X|^T |X| <= sqrt(n) cond |X^T X| left out of account
-    # by comparing with 1e-10 of the norm, far above n eps = 8e-14 of well-scaled blocks)
+    # they are timed there, and give the products of the one-pass variant to 1e-10 of the norm
+    # (n eps = 8e-14 per sum, times the cancellation of X^T X against |X|^T |X|, below 1e3)
     from paper_1110_2316_gb300 import api
     base = wl.varcoef_manufactured(n=boxes, W=8)
     pb = wl.Problem(base.mesh, base.f * n_rhs, base.g * n_rhs, base.a, base.grad_a)
