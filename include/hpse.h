@@ -340,24 +340,23 @@ hpse_status hpse_setup_block_preconditioner(hpse_mesh *m);
 /* Tile shape of the element-block preconditioner's two triangular products,
  * per degree W and precision: hpse_setup_block_preconditioner times every
  * candidate shape for the mesh's right-hand-side count on the factors it has
- * just built (variants 0-2 and 8 for >= 32 right-hand sides, 3-4 for 2..31 [in
- * FP64 4 on many large blocks only], 5-7 for one; 2 and 8 in FP32 only) and keeps
- * the fastest.  Variants
- * 2, 4 and 6 in FP32 and 3 and 5 in FP64 take both products in one pass over
- * the factor; for blocks of W >= 6 and five or more right-hand sides the FP32
- * ones split each operand into two TF32 parts, as variant 8 does, in sums of 16
- * terms (error 1.6e-7 against 64 bits at W = 8, FP32 multiply-adds 3e-7; a
- * right-hand side that is below 2^-110 throughout loses digits).  The others of
- * 0-7 are CUDA-core tiles; variant 8 runs both products on the
- * tensor cores (tcgen05, 128 rows x 64 right-hand sides per CTA, each FP32
- * operand split into two TF32 parts, three MMAs per product, FP32
- * accumulation in tensor memory).  hpse_block_tile returns the chosen
- * variant, its tile (rows x right-hand sides per CTA; a one-pass variant works
- * on all (W+1)^3 rows of a block) and, if ms is not NULL, the measured milliseconds of each of the 9 variants (0 for those not tried);
- * HPSE_ERR_NO_DATA before the set-up.  hpse_set_block_tile overrides the
- * choice (HPSE_ERR_INVALID_ARG for a variant that does not exist in that
- * precision, or variant 8 when its tiles were not built).  No counterpart in
- * the thesis. */
+ * just built (variants 0-2 and 8 for >= 32 right-hand sides, 3-4 for 2..31 (4 in
+ * FP64 on many large blocks only), 5-7 for one; 2 and 8 exist in FP32 only) and
+ * keeps the fastest.  Variants 2, 4 and 6 in FP32 and 3 and 5 in FP64 take both
+ * products in one pass over the factor; for blocks of W >= 6 and five or more
+ * right-hand sides the FP32 ones split each operand into two TF32 parts, as
+ * variant 8 does, in sums of 16 terms (error 1.6e-7 against 64 bits at W = 8,
+ * FP32 multiply-adds 3e-7; a right-hand side that is below 2^-110 throughout
+ * loses digits).  The others of 0-7 are CUDA-core tiles; variant 8 runs both
+ * products on the tensor cores (tcgen05, 128 rows x 64 right-hand sides per CTA,
+ * each FP32 operand split into two TF32 parts, three MMAs per product, FP32
+ * accumulation in tensor memory).  hpse_block_tile returns the chosen variant,
+ * its tile (rows x right-hand sides per CTA; a one-pass variant works on all
+ * (W+1)^3 rows of a block) and, if ms is not NULL, the measured milliseconds of
+ * each of the 9 variants (0 for those not tried); HPSE_ERR_NO_DATA before the
+ * set-up.  hpse_set_block_tile overrides the choice (HPSE_ERR_INVALID_ARG for a
+ * variant that does not exist in that precision, or variant 8 when its tiles
+ * were not built).  No counterpart in the thesis. */
 hpse_status hpse_block_tile(const hpse_mesh *m, int32_t W, int32_t prec, int32_t *variant, int32_t *tile_rows,
                             int32_t *tile_rhs, float *ms);
 hpse_status hpse_set_block_tile(hpse_mesh *m, int32_t W, int32_t prec, int32_t variant);
@@ -365,11 +364,12 @@ hpse_status hpse_set_block_tile(hpse_mesh *m, int32_t W, int32_t prec, int32_t v
 /* Limit of the device waits of the block products (the one-pass and the
  * tensor-core variants wait for copies and matrix instructions of their own): a
  * wait gives up after `polls` polls (0 to 2^22, the default, about a second;
- * HPSE_ERR_INVALID_ARG outside).  A product that gave up leaves NaN in its part of z; the
- * next hpse_apply_preconditioner or hpse_pcg_solve with HPSE_PRECOND_BLOCK, and
- * the solve in which it happened, return HPSE_ERR_CUDA until
- * hpse_setup_block_preconditioner is called again.  The set-up drops a variant
- * that gives up while it is timed.  Low limits are for tests of this path. */
+ * HPSE_ERR_INVALID_ARG outside).  A product that gave up leaves NaN in its part
+ * of z; the next hpse_apply_preconditioner or hpse_pcg_solve with
+ * HPSE_PRECOND_BLOCK, and the solve in which it happened, return HPSE_ERR_CUDA
+ * until hpse_setup_block_preconditioner is called again.  The set-up drops a
+ * variant that gives up while it is timed.  Low limits are for tests of this
+ * path. */
 hpse_status hpse_set_block_wait(hpse_mesh *m, int32_t polls);
 
 /* Choose the preconditioner (hpse_precond_kind).  HPSE_PRECOND_BLOCK needs a
